@@ -83,12 +83,14 @@ int encode_field_map(CUtensorMap* m, void* field_base, int st, const Geom& g, in
                      bool promote_l2 = true);
 
 // Utility kernels (k_util.cu).
-// Rows r (r = y + z ny) in [r_lo, r_hi) only (r_hi < 0: every row); the dense buffer holds those
-// rows, x fastest.
-cudaError_t launch_pack(const Geom& g, int st, const void* src, int src_dtype, void* dst_level, int field,
-                        double ref, cudaStream_t s, long long r_lo = 0, long long r_hi = -1);
-cudaError_t launch_unpack(const Geom& g, int st, const void* src_level, int field, double ref, void* dst,
-                          int dst_dtype, cudaStream_t s, long long r_lo = 0, long long r_hi = -1);
+// Dense buffers src[0 .. nf) of element type src_dtype (MMFD_DT_*) into fields field0 .. of a level
+// (and of a second level of the same layout, if given), with their periodic ghost images; refs are
+// the fields' storage references.  One launch.
+cudaError_t launch_pack(const Geom& g, int st, const void* const* src, int nf, int src_dtype, void* level, void* level2,
+                        int field0, const double* refs, cudaStream_t s);
+// The reverse: fields field0 .. of a level into dense buffers.
+cudaError_t launch_unpack(const Geom& g, int st, const void* level, int field0, int nf, const double* refs,
+                          void* const* dst, int dst_dtype, cudaStream_t s);
 // Rows [r_lo, r_hi) of all nf fields of a level to (pack) or from (unpack) nf dense buffers of
 // element type dtype (MMFD_DT_*), one launch; refs are the fields' storage references.
 cudaError_t launch_rows(const Geom& g, int st, bool pack, const void* const* bufs, int nf, int dtype, void* level,

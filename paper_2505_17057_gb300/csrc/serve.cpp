@@ -180,12 +180,11 @@ int admit(Server* s, Req* q) {
         e = cudaMemcpyAsync(s->stage, q->init.data() + (size_t)f * N * esz, (size_t)N * esz, cudaMemcpyHostToDevice,
                             s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync init");
-        for (int lv = 0; lv < (nl == 3 ? 2 : 1); ++lv) {
-            // three-level requests start from phi^{-1} := phi^0 (level index 2 = prev of cur 0)
-            void* dst = q->lev[lv == 0 ? 0 : 2];
-            e = launch_pack(q->g, q->r->st, s->stage, q->dtype, dst, f, q->r->ref[f], s->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "pack kernel");
-        }
+        // three-level requests start from phi^{-1} := phi^0 (level index 2 = prev of cur 0)
+        const void* src = s->stage;
+        e = launch_pack(q->g, q->r->st, &src, 1, q->dtype, q->lev[0], nl == 3 ? q->lev[2] : nullptr, f, &q->r->ref[f],
+                        s->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "pack kernel");
     }
     q->init.clear();
     q->init.shrink_to_fit();
@@ -728,7 +727,7 @@ int mmfd_result_fields(mmfd_server* h, unsigned long long ticket, void* const* o
     }
     for (int f = 0; f < q->g.nf; ++f) {
         void* dst = where == MMFD_HOST ? s->stage : out[f];
-        cudaError_t e = launch_unpack(q->g, q->r->st, q->lev[q->cur], f, q->r->ref[f], dst, dtype, s->stream);
+        cudaError_t e = launch_unpack(q->g, q->r->st, q->lev[q->cur], f, 1, &q->r->ref[f], &dst, dtype, s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "unpack kernel");
         if (where == MMFD_HOST) {
             e = cudaMemcpyAsync(out[f], s->stage, (size_t)N * esz, cudaMemcpyDeviceToHost, s->stream);

@@ -37,6 +37,39 @@ int level_index(const Solver* s, int level, int* idx) {
     return set_error(MMFD_ERR_ARG, "level must be 0 (t_n) or, for three-level solvers, 1 (t_{n-1})");
 }
 
+// nf dense fields (host or device) into `level` (and level2, level3 where given), a level of layout g
+// and storage st.  Device fields go in one launch per level pair; page-locked host memory is read
+// by the pack kernel itself, over the host link (one pass instead of a copy into the staging buffer
+// plus a second pass over it); other host memory is staged field by field.
+int upload(Solver* s, const Geom& g, int st, const void* const* fields, int nf, int where, int dtype, const double* refs,
+           void* level, void* level2 = nullptr, void* level3 = nullptr) {
+    for (int f = 0; f < nf; ++f)
+        if (!fields[f]) return set_error(MMFD_ERR_ARG, "null field pointer");
+    auto pack = [&](const void* const* src, int f0, int count) -> int {
+        cudaError_t e = launch_pack(g, st, src, count, dtype, level, level2, f0, refs + f0, s->stream);
+        if (e == cudaSuccess && level3) e = launch_pack(g, st, src, count, dtype, level3, nullptr, f0, refs + f0, s->stream);
+        return e == cudaSuccess ? MMFD_OK : cuda_fail(e, "pack kernel");
+    };
+    if (where == MMFD_DEVICE) return pack(fields, 0, nf);
+    int rc = ensure_stage(s);
+    if (rc != MMFD_OK) return rc;
+    const size_t bytes = (size_t)nodes(s) * (dtype == MMFD_DT_F64 ? 8 : 4);
+    for (int f = 0; f < nf; ++f) {
+        const void* src = fields[f];
+        cudaPointerAttributes pa{};
+        if (cudaPointerGetAttributes(&pa, src) == cudaSuccess && pa.type == cudaMemoryTypeHost && pa.devicePointer) {
+            src = pa.devicePointer;
+        } else {
+            cudaGetLastError();
+            cudaError_t e = cudaMemcpyAsync(s->stage, src, bytes, cudaMemcpyHostToDevice, s->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync H2D");
+            src = s->stage;
+        }
+        if ((rc = pack(&src, f, 1)) != MMFD_OK) return rc;
+    }
+    return MMFD_OK;
+}
+
 }  // namespace
 
 int solver_init_device(Solver* s) {
@@ -125,39 +158,11 @@ int solver_set_fields(Solver* s, int level, const void* const* fields, int where
     int idx;
     int rc = level_index(s, level, &idx);
     if (rc != MMFD_OK) return rc;
-    const size_t esz = dtype == MMFD_DT_F64 ? 8 : 4;
-    const size_t bytes = (size_t)nodes(s) * esz;
-    if (where == MMFD_HOST && (rc = ensure_stage(s)) != MMFD_OK) return rc;
-    for (int f = 0; f < s->g.nf; ++f) {
-        if (!fields[f]) return set_error(MMFD_ERR_ARG, "null field pointer");
-        const void* src = fields[f];
-        if (where == MMFD_HOST) {
-            // page-locked host memory is read by the pack kernel itself, over the host link (one
-            // pass instead of a copy into the staging buffer plus a second pass over it)
-            cudaPointerAttributes pa{};
-            if (cudaPointerGetAttributes(&pa, src) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
-                pa.devicePointer) {
-                src = pa.devicePointer;
-            } else {
-                cudaGetLastError();
-                cudaError_t e = cudaMemcpyAsync(s->stage, src, bytes, cudaMemcpyHostToDevice, s->stream);
-                if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync H2D");
-                src = s->stage;
-            }
-        }
-        cudaError_t e = launch_pack(s->g, s->r.st, src, dtype, s->lev[idx], f, s->r.ref[f], s->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "pack kernel");
-        if (s->nlev == 3 && level == 0) {
-            // equilibrium start: level t - dt := level t until set explicitly
-            e = launch_pack(s->g, s->r.st, src, dtype, s->lev[s->prev()], f, s->r.ref[f], s->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "pack kernel");
-        }
-        if (s->r.dirichlet && level == 0) {
-            // Dirichlet: the boundary keeps these values until mmfd_set_boundary replaces them
-            e = launch_pack(s->g, s->r.st, src, dtype, s->bnd, f, s->r.ref[f], s->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "pack kernel");
-        }
-    }
+    // three levels: the equilibrium start, level t - dt := level t until set explicitly; Dirichlet:
+    // the boundary keeps these values until mmfd_set_boundary replaces them
+    rc = upload(s, s->g, s->r.st, fields, s->g.nf, where, dtype, s->r.ref, s->lev[idx],
+                s->nlev == 3 && level == 0 ? s->lev[s->prev()] : nullptr, s->r.dirichlet && level == 0 ? s->bnd : nullptr);
+    if (rc != MMFD_OK) return rc;
     s->fields_set = true;
     if (level == 0) s->src_fresh = true;
     return MMFD_OK;
@@ -183,57 +188,15 @@ int solver_set_source(Solver* s, int level, const void* const* fields, int where
     Geom gs = s->g;
     gs.es = s->r.st == ST_F64 ? 8 : 4;
     const int sst = s->r.st == ST_F64 ? ST_F64 : ST_F32;
-    const size_t esz = dtype == MMFD_DT_F64 ? 8 : 4;
-    const size_t bytes = (size_t)nodes(s) * esz;
-    int rc;
-    if (where == MMFD_HOST && (rc = ensure_stage(s)) != MMFD_OK) return rc;
-    for (int f = 0; f < s->r.nsrc; ++f) {
-        if (!fields[f]) return set_error(MMFD_ERR_ARG, "null field pointer");
-        const void* src = fields[f];
-        if (where == MMFD_HOST) {
-            cudaPointerAttributes pa{};
-            if (cudaPointerGetAttributes(&pa, src) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
-                pa.devicePointer) {
-                src = pa.devicePointer;
-            } else {
-                cudaGetLastError();
-                cudaError_t e = cudaMemcpyAsync(s->stage, src, bytes, cudaMemcpyHostToDevice, s->stream);
-                if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync H2D");
-                src = s->stage;
-            }
-        }
-        cudaError_t e = launch_pack(gs, sst, src, dtype, s->srcbuf[idx], f, 0.0, s->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "pack kernel");
-    }
-    return MMFD_OK;
+    const double zero[4] = {0.0, 0.0, 0.0, 0.0};   // sources carry no reference
+    return upload(s, gs, sst, fields, s->r.nsrc, where, dtype, zero, s->srcbuf[idx]);
 }
 
 int solver_set_boundary(Solver* s, const void* const* fields, int where, int dtype) {
     if (!s->r.dirichlet) return set_error(MMFD_ERR_STATE, "the solver has periodic boundaries");
     if (dtype != MMFD_DT_F64 && dtype != MMFD_DT_F32) return set_error(MMFD_ERR_ARG, "dtype must be F64 or F32");
     if (where != MMFD_HOST && where != MMFD_DEVICE) return set_error(MMFD_ERR_ARG, "where must be HOST or DEVICE");
-    const size_t bytes = (size_t)nodes(s) * (dtype == MMFD_DT_F64 ? 8 : 4);
-    int rc;
-    if (where == MMFD_HOST && (rc = ensure_stage(s)) != MMFD_OK) return rc;
-    for (int f = 0; f < s->g.nf; ++f) {
-        if (!fields[f]) return set_error(MMFD_ERR_ARG, "null field pointer");
-        const void* src = fields[f];
-        if (where == MMFD_HOST) {
-            cudaPointerAttributes pa{};
-            if (cudaPointerGetAttributes(&pa, src) == cudaSuccess && pa.type == cudaMemoryTypeHost &&
-                pa.devicePointer) {
-                src = pa.devicePointer;
-            } else {
-                cudaGetLastError();
-                cudaError_t e = cudaMemcpyAsync(s->stage, src, bytes, cudaMemcpyHostToDevice, s->stream);
-                if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync H2D");
-                src = s->stage;
-            }
-        }
-        cudaError_t e = launch_pack(s->g, s->r.st, src, dtype, s->bnd, f, s->r.ref[f], s->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "pack kernel");
-    }
-    return MMFD_OK;
+    return upload(s, s->g, s->r.st, fields, s->g.nf, where, dtype, s->r.ref, s->bnd);
 }
 
 void solver_launch_args(Solver* s, LaunchArgs& a) {
@@ -356,17 +319,19 @@ int solver_get_fields(Solver* s, int level, void* const* out, int where, int dty
     const size_t esz = dtype == MMFD_DT_F64 ? 8 : 4;
     const size_t bytes = (size_t)nodes(s) * esz;
     if (where == MMFD_HOST && (rc = ensure_stage(s)) != MMFD_OK) return rc;
-    for (int f = 0; f < s->g.nf; ++f) {
+    for (int f = 0; f < s->g.nf; ++f)
         if (!out[f]) return set_error(MMFD_ERR_ARG, "null field pointer");
-        void* dst = where == MMFD_HOST ? s->stage : out[f];
-        cudaError_t e = launch_unpack(s->g, s->r.st, s->lev[idx], f, s->r.ref[f], dst, dtype, s->stream);
+    if (where == MMFD_DEVICE) {
+        cudaError_t e = launch_unpack(s->g, s->r.st, s->lev[idx], 0, s->g.nf, s->r.ref, out, dtype, s->stream);
+        return e == cudaSuccess ? MMFD_OK : cuda_fail(e, "unpack kernel");
+    }
+    for (int f = 0; f < s->g.nf; ++f) {
+        cudaError_t e = launch_unpack(s->g, s->r.st, s->lev[idx], f, 1, s->r.ref + f, &s->stage, dtype, s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "unpack kernel");
-        if (where == MMFD_HOST) {
-            e = cudaMemcpyAsync(out[f], s->stage, bytes, cudaMemcpyDeviceToHost, s->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync D2H");
-            e = cudaStreamSynchronize(s->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-        }
+        e = cudaMemcpyAsync(out[f], s->stage, bytes, cudaMemcpyDeviceToHost, s->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync D2H");
+        e = cudaStreamSynchronize(s->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     }
     return MMFD_OK;
 }
