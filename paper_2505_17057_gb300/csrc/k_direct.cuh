@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "launch.cuh"
 #include "stencil.cuh"
 
 namespace mmfd {
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(256) k_direct(Geom g, const void* __restrict__
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     if (x >= g.nx || y >= g.ny) return;
+    chain_wait();
     direct_node<LAT, PDE, LEVELS, ST>(g, in0v, in1v, outv, cf, ex, x, y, z);
 }
 
@@ -142,9 +144,8 @@ cudaError_t launch_direct(const LaunchArgs& a) {
     using T = typename Storage<ST>::T;
     dim3 block(64, 4, 1);
     dim3 grid((a.g.nx + block.x - 1) / block.x, (a.g.ny + block.y - 1) / block.y, a.g.nz);
-    k_direct<LAT, PDE, LEVELS, ST><<<grid, block, 0, a.stream>>>(a.g, a.in0, a.in1, a.out,
+    return launch_chained(k_direct<LAT, PDE, LEVELS, ST>, grid, block, 0, a.stream, a.chained, a.g, a.in0, a.in1, a.out,
                                                                   *static_cast<const Coef<T>*>(a.coef), a.ex);
-    return cudaGetLastError();
 }
 
 template <int LAT, int PDE, int LEVELS, int ST, int SRC>
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(256) k_direct_src(Geom g, const void* __restri
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     if (x >= g.nx || y >= g.ny) return;
+    chain_wait();
     direct_node<LAT, PDE, LEVELS, ST, SRC>(g, in0v, in1v, outv, cf, ex, x, y, z, &sa);
 }
 
@@ -168,9 +170,8 @@ cudaError_t launch_direct_src(const LaunchArgs& a) {
     sa.w = *static_cast<const SrcCoef<T>*>(a.src_coef);
     dim3 block(64, 4, 1);
     dim3 grid((a.g.nx + block.x - 1) / block.x, (a.g.ny + block.y - 1) / block.y, a.g.nz);
-    k_direct_src<LAT, PDE, LEVELS, ST, SRC><<<grid, block, 0, a.stream>>>(
+    return launch_chained(k_direct_src<LAT, PDE, LEVELS, ST, SRC>, grid, block, 0, a.stream, a.chained, 
         a.g, a.in0, a.in1, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, sa);
-    return cudaGetLastError();
 }
 
 }  // namespace mmfd

@@ -453,8 +453,10 @@ __global__ void __launch_bounds__(NW * 32) k_march2d(const __grid_constant__ Tma
         fence_mbar_init();
 #pragma unroll
         for (int q = 0; q < NIN; ++q) tma_prefetch_desc(&maps.m[q]);
-        for (int k = 0; k < NSTAGE; ++k) issue_next();
     }
+    chain_wait();
+    if (lane == 0)
+        for (int k = 0; k < NSTAGE; ++k) issue_next();
     __syncwarp();
 
     // Accumulators of the output rows around the staged input rows: with RPS = 1, acc0/1/2 are
@@ -793,9 +795,8 @@ cudaError_t launch_march2d_t(const LaunchArgs& a) {
         sa.s[1] = static_cast<const T*>(LEVELS == 3 ? a.src[1] : a.src[0]);
         sa.w = *static_cast<const SrcCoef<T>*>(a.src_coef);
     }
-    kern<<<grid, NW * 32, smem, a.stream>>>(*a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
+    return launch_chained(kern, grid, NW * 32, smem, a.stream, a.chained, *a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
                                              nitems, a.err, sa);
-    return cudaGetLastError();
 }
 
 // The same with the stochastic-rounding choice made per launch (BF16 storage: an instantiation

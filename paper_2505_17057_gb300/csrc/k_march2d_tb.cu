@@ -164,8 +164,10 @@ __global__ void __launch_bounds__(NW * 32) k_march2d_tb(const __grid_constant__ 
         for (int s = 0; s < NSTAGE; ++s) mbar_init(&full[s], 1);
         fence_mbar_init();
         tma_prefetch_desc(&maps.m[0]);
-        for (int k = 0; k < NSTAGE; ++k) issue_next();
     }
+    chain_wait();
+    if (lane == 0)
+        for (int k = 0; k < NSTAGE; ++k) issue_next();
     __syncwarp();
 
     // accumulators: level t holds rows (P, C, N) = (r-1, r, r+1) of its current input row r.
@@ -371,9 +373,8 @@ cudaError_t launch_tb(const LaunchArgs& a) {
         rhs = static_cast<const S*>(a.src[0]);
         jw = static_cast<const SrcCoef<T>*>(a.src_coef)->W0[0];
     }
-    kern<<<grid, NW * 32, smem, a.stream>>>(*a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
+    return launch_chained(kern, grid, NW * 32, smem, a.stream, a.chained, *a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
                                              nitems, a.err, rhs, jw);
-    return cudaGetLastError();
 }
 
 template <int LAT, int PDE, int ST, bool JAC = false>

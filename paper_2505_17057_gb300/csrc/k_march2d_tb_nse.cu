@@ -152,8 +152,10 @@ __global__ void __launch_bounds__(NW * 32) k_march2d_tb_nse(const __grid_constan
         fence_mbar_init();
 #pragma unroll
         for (int f = 0; f < NF; ++f) tma_prefetch_desc(&maps.m[f]);
-        for (int k = 0; k < NSTAGE; ++k) issue_next();
     }
+    chain_wait();
+    if (lane == 0)
+        for (int k = 0; k < NSTAGE; ++k) issue_next();
     __syncwarp();
 
     // accumulators: level t holds rows (P, C, N) = (r-1, r, r+1) of its current input row r
@@ -301,9 +303,8 @@ cudaError_t launch_tbn_t(const LaunchArgs& a) {
     const int nitems = strips * ((a.g.ny + H - 1) / H);
     const int blocks_needed = (nitems + NW - 1) / NW;
     const int grid = blocks_needed < resident ? blocks_needed : resident;
-    kern<<<grid, NW * 32, smem, a.stream>>>(*a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
+    return launch_chained(kern, grid, NW * 32, smem, a.stream, a.chained, *a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
                                              nitems, a.err);
-    return cudaGetLastError();
 }
 
 // stochastic rounding chosen per launch: BF16 has a kernel without and one with the rounding code

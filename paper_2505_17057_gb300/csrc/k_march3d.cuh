@@ -106,6 +106,7 @@ __global__ void __launch_bounds__((TY + 1) * 32, (LEAN != LEAN_NONE && TY <= 4) 
         for (int q = 0; q < NIN; ++q) tma_prefetch_desc(&maps.m[q]);
     }
     __syncthreads();
+    chain_wait();
 
     if (warp == TY) {
         // ---------------------------------------------------------------- producer warp
@@ -439,9 +440,8 @@ cudaError_t launch_march3d_t(const LaunchArgs& a) {
         sa.s[1] = static_cast<const T*>(LEVELS == 3 ? a.src[1] : a.src[0]);
         sa.w = *static_cast<const SrcCoef<T>*>(a.src_coef);
     }
-    kern<<<grid, THREADS, smem, a.stream>>>(*a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
+    return launch_chained(kern, grid, THREADS, smem, a.stream, a.chained, *a.maps, a.g, a.out, *static_cast<const Coef<T>*>(a.coef), a.ex, H,
                                             nitems, a.err, sa);
-    return cudaGetLastError();
 }
 
 // The same with the stochastic-rounding choice made per launch (see launch_march2d_sr).

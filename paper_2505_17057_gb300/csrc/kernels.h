@@ -30,6 +30,7 @@ struct LaunchArgs {
     int* err;             // device error flag (bounded waits that ran out)
     const void* src[2];   // source levels t, t - dt (solvers with source terms; else null)
     const void* src_coef; // SrcCoef<double> or SrcCoef<float> matching the storage type
+    bool chained = false; // a step of a chain on one stream: launched to overlap its predecessor's end (launch.cuh)
 };
 using LaunchFn = cudaError_t (*)(const LaunchArgs&);
 

@@ -213,6 +213,7 @@ void solver_launch_args(Solver* s, LaunchArgs& a) {
     a.H = s->H;
     a.err = s->d_flag;
     a.maps = nullptr;
+    a.chained = s->chained;
     a.src[0] = s->r.src ? s->srcbuf[s->src_i0] : nullptr;
     a.src[1] = s->r.src ? s->srcbuf[s->src_i1] : nullptr;
     a.src_coef = s->r.st == ST_F64 ? static_cast<const void*>(&s->r.sd) : static_cast<const void*>(&s->r.sf);
@@ -235,6 +236,10 @@ void solver_launch_args(Solver* s, LaunchArgs& a) {
 
 int solver_step(Solver* s, long long nsteps) {
     if (!s->fields_set) return set_error(MMFD_ERR_STATE, "set the fields before stepping");
+    // steps of a captured stream keep the plain dependencies of the capture
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(s->stream, &cap) != cudaSuccess) cudaGetLastError();
+    s->chained = cap == cudaStreamCaptureStatusNone;
     if (s->r.theta_on) {
         // Eq. (GCN): rhs = ((1 - theta) I + theta E) phi^n, then r.sweeps Jacobi sweeps from
         // x = phi^n, each into the spare level buffer

@@ -36,6 +36,7 @@ struct Solver {
     int tile_rows = 0;  // 3D marching kernels: rows of the CTA tile (mmfd_info_t::tile_rows)
     int* d_flag = nullptr;                       // device error flag written by kernels
     bool fields_set = false;
+    bool chained = false;                        // this mmfd_step call launches its steps chained (launch.cuh)
     bool use_tma = false;                        // kernel family consumes tensor maps
     int lean = 0;                                // LEAN_* variant of the marching kernel in use
     CUtensorMap tmaps[3][4];                     // per level buffer, per field
