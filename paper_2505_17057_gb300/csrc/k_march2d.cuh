@@ -59,14 +59,137 @@ __device__ __forceinline__ void stg4(void* p, const typename Storage<ST>::S s[4]
     }
 }
 
-// Store four consecutive nodes xb .. xb+3 (xb a multiple of 4) of row y, plane z, together with
-// their periodic ghost images: the x ghosts within g.gx of either x edge, the ghost row of
-// y = 0 / ny - 1 and, in 3D, the ghost plane of z = 0 / nz - 1 (with all combinations).  Nodes
-// outside [0, nx) are skipped.  Straight-line predicated stores, no local arrays: the warps that
-// own edge strips and rows must not fall behind the others.
-// (The four values come as scalars: an array passed by address to an out-of-line function would
-// have to live in local memory in the caller, on every row, for every lane.)
-template <int DIM, int ST>
+// The output store of the marching kernels.  A lane writes its four nodes xb .. xb+3 (xb a
+// multiple of 4) and their periodic ghost images -- the x ghosts within g.gx of either x edge, the
+// ghost row of y = 0 / ny - 1 and, in 3D, the ghost plane of z = 0 / nz - 1, with all combinations
+// -- with predicated stores only, all 32 lanes following the same control flow: a lane that
+// branched off alone onto an edge path made its whole warp run about three times slower on every
+// row (measured per warp with %globaltimer), and the warps owning the edge strips then set the
+// length of the launch.  What depends only on the lane's columns is worked out once per work item
+// (init).  Whole vectors cover the usual grids; where the lane's nodes straddle x = nx or the
+// images are not vector-aligned (nx not a multiple of 4), the warps of the edge strips add
+// predicated single stores, again all lanes together (a divergent scalar path for those lanes ran
+// 4095 x 4096 NSE FP32 steps at 137 us against 85 for 4096 x 4096).
+// ONES false: the caller knows that nx is a multiple of 4, and no lane has single stores.
+template <int DIM, int ST, bool ONES = true>
+struct EdgeStore {
+    using S = typename Storage<ST>::S;
+    static constexpr int OX = 16 / (int)sizeof(S);   // ghost block width (elements)
+    // what the lane writes: single stores, a bit per node: own slot (0-3), image at x + nx (4-7), at
+    // x - nx (8-11); and whole vectors: its four nodes, all output nodes inside [0, nx) (kIn), the x
+    // ghost block at x + nx (kLo), at x - nx (kHi); kOnes: some lane of the warp has single stores
+    enum { kIn = 1 << 12, kLo = 1 << 13, kHi = 1 << 14, kOnes = 1 << 15, kAny = 1 << 16 };
+    int m = 0;
+
+    // all 32 lanes, once per item
+    __device__ __forceinline__ void init(const Geom& g, int xb, bool valid) {
+        const bool in = valid && xb >= 0 && xb + 3 < g.nx;
+        bool lo, hi;
+        if constexpr (OX >= 4) {
+            // FP32 / BF16: the lane's nodes are one 16- or 8-byte piece of the block; the image at
+            // x -+ nx is vector-aligned only when nx is a multiple of 4
+            const bool al = (g.nx & 3) == 0;
+            lo = in && al && xb + 3 < OX;
+            hi = in && al && xb >= g.nx - OX;
+        } else {
+            // FP64: the block is two doubles, the first or last half of the lane
+            lo = in && xb == 0 && (g.nx & 1) == 0;
+            hi = in && xb + 4 == g.nx && (g.nx & 1) == 0;
+        }
+        m = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int x = xb + k;
+            if (valid && x >= 0 && x < g.nx) {
+                if (!in) m |= 1 << k;
+                if (!lo && x < g.gx) m |= 16 << k;
+                if (!hi && x >= g.nx - g.gx) m |= 256 << k;
+            }
+        }
+        const bool ones = __any_sync(0xffffffffu, m != 0), any = __any_sync(0xffffffffu, m != 0 || lo || hi);
+        m |= (in ? kIn : 0) | (lo ? kLo : 0) | (hi ? kHi : 0) | (ones ? kOnes : 0) | (any ? kAny : 0);
+    }
+
+    // The lane's four nodes of every field (field f at out + f fs, its values from val(f, sv)) of row y,
+    // plane z; all 32 lanes (warp-uniform y, z).  Rows and planes at an edge are stored again at their
+    // images: in 2D by one instance of the stores in a loop that runs once elsewhere, in 3D out of line.
+    // (Three inlined instances took 20 to 60 more registers: nse2d_4096 BF16, three steps per launch, 48.8 us
+    // per step against 41.4.  The loop in 3D: cde3d_512 FP32 247 us against 182.)
+    template <int NF, typename F>
+    __device__ __forceinline__ void put(S* out, long long fs, const Geom& g, int xb, int y, int z, F&& val) const {
+        S sv[NF][4];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) val(f, sv[f]);
+        S* const p = out + g.at(xb, y, z);
+        S* q = p;
+        if constexpr (DIM == 2) {
+            const bool edge = y == 0 || y == g.ny - 1;
+            int img = -1;   // images left: beyond the far edge (1), the near one (2)
+            for (;;) {
+                put_fields<NF>(q, fs, g.nx, sv);
+                if (!edge) break;
+                if (img < 0) img = (y == 0 ? 1 : 0) | (y == g.ny - 1 ? 2 : 0);
+                if (img == 0) break;
+                q = p + (long long)(img & 1 ? g.ny : -g.ny) * g.py;
+                img &= img - 1;
+            }
+        } else {
+            put_fields<NF>(p, fs, g.nx, sv);
+            if (y == 0 || y == g.ny - 1 || z == 0 || z == g.nz - 1) {
+                const int img = (y == 0 ? 1 : 0) | (y == g.ny - 1 ? 2 : 0) | (z == 0 ? 4 : 0) | (z == g.nz - 1 ? 8 : 0);
+#pragma unroll
+                for (int f = 0; f < NF; ++f)
+                    put_images(p + f * fs, g.nx, m, img, (long long)g.ny * g.py, (long long)g.nz * g.pz, sv[f][0], sv[f][1],
+                               sv[f][2], sv[f][3]);
+            }
+        }
+    }
+    template <int NF>
+    __device__ __forceinline__ void put_fields(S* q, long long fs, int nx, const S (&sv)[NF][4]) const {
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+            if (m & kIn) stg4<ST>(q + f * fs, sv[f]);
+        if (NF == 1 || (m & kAny)) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f) put_x(q + f * fs, nx, m, sv[f]);
+        }
+    }
+    // img: bits y = 0, y = ny - 1, z = 0, z = nz - 1; dy, dz: the grid's extents in the layout.  The values come
+    // as scalars: an array passed by address would have to live in local memory in the caller.
+    __device__ static __noinline__ void put_images(S* p, int nx, int m, int img, long long dy, long long dz, S s0, S s1, S s2,
+                                                   S s3) {
+        const S sv[4] = {s0, s1, s2, s3};
+        for (int c = 1; c < 9; ++c) {
+            const int cy = c % 3, cz = c / 3;   // 0: itself, 1: the image beyond the far edge, 2: beyond the near one
+            if ((cy != 0 && !(img & cy)) || (cz != 0 && !(img & (cz << 2)))) continue;
+            S* q = p + (cy == 0 ? 0 : cy == 1 ? dy : -dy) + (cz == 0 ? 0 : cz == 1 ? dz : -dz);
+            if (m & kIn) stg4<ST>(q, sv);
+            put_x(q, nx, m, sv);
+        }
+    }
+    // what a row holds beyond the lane's own vector: x ghost blocks and single stores
+    __device__ static __forceinline__ void put_x(S* p, int nx, int m, const S (&sv)[4]) {
+        if constexpr (OX >= 4) {
+            if (m & kLo) stg4<ST>(p + nx, sv);
+            if (m & kHi) stg4<ST>(p - nx, sv);
+        } else {
+            if (m & kLo) *reinterpret_cast<double2*>(p + nx) = make_double2(sv[0], sv[1]);
+            if (m & kHi) *reinterpret_cast<double2*>(p + 2 - nx) = make_double2(sv[2], sv[3]);
+        }
+        if (ONES && (m & kOnes)) {   // (warp-uniform)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (m & (1 << k)) p[k] = sv[k];
+                if (m & (16 << k)) p[k + nx] = sv[k];
+                if (m & (256 << k)) p[k - nx] = sv[k];
+            }
+        }
+    }
+};
+
+// Four consecutive nodes xb .. xb + 3 of row y, plane z, with all their periodic images; nodes outside
+// [0, nx) are skipped.
+template <int ST>
 __device__ __noinline__ void store4_ghosted(typename Storage<ST>::S* f, const Geom g, int xb, int y, int z,
                                             typename Storage<ST>::S s0, typename Storage<ST>::S s1,
                                             typename Storage<ST>::S s2, typename Storage<ST>::S s3) {
@@ -101,45 +224,34 @@ __device__ __noinline__ void store4_ghosted(typename Storage<ST>::S* f, const Ge
         if (yhi) put_row(-1, zz);
     };
     put_plane(z);
-    if constexpr (DIM == 3) {
-        if (z == 0) put_plane(g.nz);
-        if (z == g.nz - 1) put_plane(-1);
-    }
+    if (z == 0) put_plane(g.nz);
+    if (z == g.nz - 1) put_plane(-1);
 }
 
-// The output store of the marching kernels.  A lane writes its four nodes xb .. xb+3 (xb a
-// multiple of 4) and their periodic ghost images -- the ghost row of y = 0 / ny - 1 and the
-// whole-vector x ghost blocks -- with predicated stores only, all 32 lanes following the same
-// control flow: a lane that branched off alone onto an edge path made its whole warp run about
-// three times slower on every row (measured per warp with %globaltimer), and the warps owning
-// the edge strips then set the length of the launch.  What depends only on the lane's columns
-// is worked out once per work item (init); the cases vectors cannot cover (z edge planes,
-// ny == 1, vectors straddling x = nx, x ghosts when nx is not a multiple of 4) take
-// store4_ghosted under a warp-uniform branch.
-template <int DIM, int ST>
-struct EdgeStore {
+// EdgeStore for k_march3d's kernels of several fields, one field at a time.  These (the NSE at 96 registers
+// a thread, bound by instruction issue) run best on conditions that stay in predicate registers,
+// each field stored before the next is formed, and one call per lane and field for the stores no
+// aligned grid needs: a step of nse3d_512 BF16 takes 990 us so and 1024 - 1190 us in the forms above.
+template <int ST>
+struct EdgeStore3 {
     using S = typename Storage<ST>::S;
     static constexpr int OX = 16 / (int)sizeof(S);   // ghost block width (elements)
     bool in = false;      // the lane's four nodes are output nodes inside [0, nx)
     bool lo = false;      // writes the x ghost block at x + nx as a vector
     bool hi = false;      // writes the x ghost block at x - nx as a vector
-    bool xrare = false;   // needs the general path (partial vector, scalar x ghosts)
+    bool xrare = false;   // needs store4_ghosted (partial vector, scalar x ghosts)
     bool wrare = false;   // some lane of the warp does (warp-uniform)
 
-    // all 32 lanes, once per item
     __device__ __forceinline__ void init(const Geom& g, int xb, bool valid) {
         in = valid && xb >= 0 && xb + 3 < g.nx;
         const bool part = valid && !in && xb < g.nx && xb + 3 >= 0;
         bool xdone;
         if constexpr (OX >= 4) {
-            // FP32 / BF16: the lane's nodes are one 16- or 8-byte piece of the block; the image at
-            // x -+ nx is vector-aligned only when nx is a multiple of 4
             const bool al = (g.nx & 3) == 0;
             lo = in && al && xb + 3 < OX;
             hi = in && al && xb >= g.nx - OX;
             xdone = !(in && (xb < g.gx || xb + 3 >= g.nx - g.gx)) || lo || hi;
         } else {
-            // FP64: the block is two doubles, the first or last half of the lane
             lo = in && xb == 0 && (g.nx & 1) == 0;
             hi = in && xb + 4 == g.nx;
             xdone = (!(in && xb < g.gx) || lo) && (!(in && xb + 3 >= g.nx - g.gx) || hi);
@@ -147,8 +259,6 @@ struct EdgeStore {
         xrare = part || !xdone;
         wrare = __any_sync(0xffffffffu, xrare);
     }
-
-    // all 32 lanes (warp-uniform y, z)
     __device__ __forceinline__ void put(S* f, const Geom& g, int xb, int y, int z, const S (&sv)[4]) const {
         S* p = f + g.at(xb, y, z);
         if (in) stg4<ST>(p, sv);
@@ -168,9 +278,9 @@ struct EdgeStore {
                 if (hi && ydup) *reinterpret_cast<double2*>(p + 2 - g.nx + dy) = make_double2(sv[2], sv[3]);
             }
         }
-        const bool plane_rare = g.ny == 1 || (DIM == 3 && (z == 0 || z == g.nz - 1));
+        const bool plane_rare = g.ny == 1 || z == 0 || z == g.nz - 1;
         if (wrare || plane_rare) {
-            if (xrare || (plane_rare && (in || xrare))) store4_ghosted<DIM, ST>(f, g, xb, y, z, sv[0], sv[1], sv[2], sv[3]);
+            if (xrare || (plane_rare && (in || xrare))) store4_ghosted<ST>(f, g, xb, y, z, sv[0], sv[1], sv[2], sv[3]);
         }
     }
 };
@@ -635,24 +745,17 @@ __global__ void __launch_bounds__(NW * 32) k_march2d(const __grid_constant__ Tma
     };
     auto store_row = [&](int yo, int xb, const T (&acc)[LN][NF], const T (&add)[4]) {
         const long long nb = (long long)yo * g.nx;
+        es.template put<NF>(out, g.fs, g, xb, yo, 0, [&](int f, S (&sv)[4]) {
 #pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            S* fo = out + (size_t)f * g.fs;
-#pragma unroll
-            for (int k4 = 0; k4 < LN; k4 += 4) {
-                S sv[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const unsigned rnd = sr_on<SRM>(ex) ? sr_bits(ex.seed, ex.step, nb + xb + k4 + k, f) : 0u;
-                    T v = acc[k4 + k][f];
-                    if constexpr (SRC != 0) {
-                        if (f == 0) v += add[k];
-                    }
-                    sv[k] = kpack<ST, PDE>(v, cf.ref[f], rnd);
+            for (int k = 0; k < 4; ++k) {
+                const unsigned rnd = sr_on<SRM>(ex) ? sr_bits(ex.seed, ex.step, nb + xb + k, f) : 0u;
+                T v = acc[k][f];
+                if constexpr (SRC != 0) {
+                    if (f == 0) v += add[k];
                 }
-                es.put(fo, g, xb + k4, yo, 0, sv);
+                sv[k] = kpack<ST, PDE>(v, cf.ref[f], rnd);
             }
-        }
+        });
     };
 
     for (int item = wid; item < nitems && !failed; item += wstride) {
@@ -764,6 +867,9 @@ cudaError_t launch_march2d_t(const LaunchArgs& a) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
         if (e != cudaSuccess) return e;
+        // The plain FP32 linear step is bound by DRAM, and fewer concurrent row streams are easier on it:
+        // at 8192^2 (7 CTAs fit an SM) 116 us at 7, 113 at 5, 98 at 4, 90 at 3, 117 at 2.
+        if (PDE == PDE_LCDE && ST == ST_F32 && LEVELS == 2 && SRC == 0 && per_sm > 3) per_sm = 3;
         resident = (per_sm > 0 ? per_sm : 1) * sms;
     }
     constexpr int COLS = 32 * LN;

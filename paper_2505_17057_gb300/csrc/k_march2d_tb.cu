@@ -94,8 +94,18 @@ __device__ __forceinline__ void tb_push_row(const Coef<T>& cf, const T (&raw)[LN
     });
 }
 
+// CTAs per SM the register allocation aims at.  Left to itself the compiler keeps the rare image stores'
+// addresses in registers: 143 for four levels of the FP32 NCDE (three CTAs against five at 96), 152 for
+// the four-sweep Jacobi kernel (theta2d_4096 415 us per step against 376 at four CTAs).  Five levels do
+// not fit 96 registers (lcde2d_8192 BF16 48.5 us per step with 60 bytes spilled).
+constexpr int tb_min_ctas(int pde, int st, int tt, bool jac) {
+    if (st == ST_F64) return jac ? 3 : 4;
+    if (jac || tt == 5) return 4;
+    return tt == 2 || (pde == PDE_LCDE && tt == 3 && st == ST_F32) ? 6 : 5;
+}
+
 template <int LAT, int PDE, int ST, int TT, int NW, int NSTAGE, bool JAC>
-__global__ void __launch_bounds__(NW * 32) k_march2d_tb(const __grid_constant__ TmapSet maps, Geom g,
+__global__ void __launch_bounds__(NW * 32, tb_min_ctas(PDE, ST, TT, JAC)) k_march2d_tb(const __grid_constant__ TmapSet maps, Geom g,
                                                         void* __restrict__ outv, Coef<typename Storage<ST>::T> cf,
                                                         StepExtra ex, int H, int nitems, int* __restrict__ err,
                                                         const typename Storage<ST>::S* __restrict__ rhs,
@@ -249,13 +259,13 @@ __global__ void __launch_bounds__(NW * 32) k_march2d_tb(const __grid_constant__ 
         const int yo = y0 - 2 * TT + i;
         if (i >= 2 * TT && i < hrows + 2 * TT) {   // warp-uniform; lanes 0 and 31 hold no output
             const long long nb = (long long)yo * g.nx;
-            S sv[4];
+            es.template put<1>(out, g.fs, g, xb, yo, 0, [&](int, S (&sv)[4]) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const unsigned rnd = ex.sr ? sr_bits(ex.seed, ex.step, nb + xb + k, 0) : 0u;
-                sv[k] = kpack<ST, PDE>(raw[1 + k], cf.ref[0], rnd);
-            }
-            es.put(out, g, xb, yo, 0, sv);
+                for (int k = 0; k < 4; ++k) {
+                    const unsigned rnd = ex.sr ? sr_bits(ex.seed, ex.step, nb + xb + k, 0) : 0u;
+                    sv[k] = kpack<ST, PDE>(raw[1 + k], cf.ref[0], rnd);
+                }
+            });
         }
     };
 

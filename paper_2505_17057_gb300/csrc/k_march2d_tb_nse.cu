@@ -187,16 +187,13 @@ __global__ void __launch_bounds__(NW * 32) k_march2d_tb_nse(const __grid_constan
         const int yo = y0 - 2 * TT + i;
         if (i >= 2 * TT && i < hrows + 2 * TT) {   // warp-uniform; lanes 0 and 31 hold no output
             const long long nb = (long long)yo * g.nx;
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                S sv[4];
+            es.template put<NF>(out, g.fs, g, xb, yo, 0, [&](int f, S (&sv)[4]) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const unsigned rnd = sr_on<SRM>(ex) ? sr_bits(ex.seed, ex.step, nb + xb + k, f) : 0u;
                     sv[k] = kpack<ST, PDE>(raw[1 + k][f], cf.ref[f], rnd);
                 }
-                es.put(out + (size_t)f * g.fs, g, xb, yo, 0, sv);
-            }
+            });
         }
     };
 

@@ -26,11 +26,19 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// The lean NSE variants with 4-row tiles are held to four CTAs per SM (96 registers): on nse3d_512
-// FP32 that ran 136 GLUPS against 129 at three CTAs (119 registers).  With 16-row tiles a CTA of
-// 17 warps fills the SM on its own.
-template <int LAT, int PDE, int LEVELS, int ST, int TY, int NSTAGE, int SRC = 0, int LEAN = LEAN_NONE, int SRM = 2>
-__global__ void __launch_bounds__((TY + 1) * 32, (LEAN != LEAN_NONE && TY <= 4) ? 4 : 1) k_march3d(const __grid_constant__ TmapSet maps, Geom g,
+// CTAs per SM the register allocation aims at.  The lean NSE variants with 4-row tiles: four (96 registers);
+// on nse3d_512 FP32 that ran 136 GLUPS against 129 at three CTAs (119 registers).  With 16-row tiles a
+// CTA of 17 warps fills the SM on its own.  The linear stencil's tiles of 8 rows: two (96 registers);
+// at 100 registers one CTA of 9 warps was left of an SM's 16 (a scheduler holds four such warps), and
+// cde3d_512 BF16 ran 281 us a step.  Three-level BF16 NCDE: the same step at 96 registers.
+constexpr int march3d_min_ctas(int pde, int levels, int st, int ty, int lean) {
+    if (lean != LEAN_NONE) return ty <= 4 ? 4 : 1;
+    if (pde == PDE_LCDE) return st != ST_F64 ? 2 : 1;
+    return pde == PDE_NCDE && levels == 3 && st == ST_BF16 ? 4 : 1;
+}
+
+template <int LAT, int PDE, int LEVELS, int ST, int TY, int NSTAGE, int SRC = 0, int LEAN = LEAN_NONE, int SRM = 2, bool ONES = true>
+__global__ void __launch_bounds__((TY + 1) * 32, SRC != 0 ? 1 : march3d_min_ctas(PDE, LEVELS, ST, TY, LEAN)) k_march3d(const __grid_constant__ TmapSet maps, Geom g,
                                                            void* __restrict__ outv, Coef<typename Storage<ST>::T> cf,
                                                            StepExtra ex, int H, int nitems, int* __restrict__ err,
                                                            const __grid_constant__ SrcParam<typename Storage<ST>::T, SRC> sa) {
@@ -139,7 +147,7 @@ __global__ void __launch_bounds__((TY + 1) * 32, (LEAN != LEAN_NONE && TY <= 4) 
 
     // -------------------------------------------------------------------- consumer warps
     T accP[LN][NF], accC[LN][NF], accN[LN][NF];
-    EdgeStore<3, ST> es;
+    std::conditional_t<(NF > 1), EdgeStore3<ST>, EdgeStore<3, ST, ONES>> es;
     S* out = static_cast<S*>(outv);
     long long k = 0;
     bool failed = false;
@@ -324,9 +332,7 @@ __global__ void __launch_bounds__((TY + 1) * 32, (LEAN != LEAN_NONE && TY <= 4) 
                 const long long nb = ((long long)zo * g.ny + y) * g.nx;
                 [[maybe_unused]] T add[4];
                 if constexpr (SRC != 0) source_quad<LAT, SRC, LEVELS, T>(g, sa, y, zo, xb, add);
-#pragma unroll
-                for (int f = 0; f < NF; ++f) {
-                    S sv[4];
+                auto values = [&](int f, S (&sv)[4]) {
 #pragma unroll
                     for (int n = 0; n < 4; ++n) {
                         const unsigned rnd = sr_on<SRM>(ex) ? sr_bits(ex.seed, ex.step, nb + xb + n, f) : 0u;
@@ -336,8 +342,16 @@ __global__ void __launch_bounds__((TY + 1) * 32, (LEAN != LEAN_NONE && TY <= 4) 
                         }
                         sv[n] = kpack<ST, PDE>(v, cf.ref[f], rnd);
                     }
-                    S* fo = out + (size_t)f * g.fs;
-                    es.put(fo, g, xb, y, zo, sv);
+                };
+                if constexpr (NF == 1) {
+                    es.template put<1>(out, g.fs, g, xb, y, zo, values);
+                } else {
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) {
+                        S sv[4];
+                        values(f, sv);
+                        es.put(out + (size_t)f * g.fs, g, xb, y, zo, sv);
+                    }
                 }
             }
 #pragma unroll
@@ -387,18 +401,31 @@ cudaError_t launch_march3d_t(const LaunchArgs& a) {
     constexpr int NF = pde_nf(PDE, LAT);
     constexpr size_t smem = march3d_smem<ST, LEVELS, NF, TY, NSTAGE>();
     constexpr int THREADS = (TY + 1) * 32;
+    // The linear stencil has a second instance without the single stores, for nx a multiple of 4: they cost the
+    // other one a quarter of its time (256^3 FP32 32.2 us against 26.2).
+    constexpr bool kAligned = PDE == PDE_LCDE && SRC == 0;
+    const bool aligned = kAligned && a.g.nx % 4 == 0;
     auto kern = k_march3d<LAT, PDE, LEVELS, ST, TY, NSTAGE, SRC, LEAN, SRM>;
-    static int resident = 0;
-    if (resident == 0) {
+    if constexpr (kAligned) {
+        if (aligned) kern = k_march3d<LAT, PDE, LEVELS, ST, TY, NSTAGE, SRC, LEAN, SRM, false>;
+    }
+    static int resident_of[2] = {0, 0}, sms = 0, l2 = 0;
+    int& fit = resident_of[aligned];
+    if (fit == 0) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
+        int per_sm = 0, dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);
         if (e != cudaSuccess) return e;
-        resident = (per_sm > 0 ? per_sm : 1) * sms;
+        fit = (per_sm > 0 ? per_sm : 1) * sms;
     }
+    // Two FP32 levels larger than L2 stream through DRAM, which fewer concurrent plane streams suit better:
+    // 512^3 174 us with two CTAs per SM against 215 with three; 256^3, in L2, 28.5 against 26.1.
+    const bool streams = kAligned && ST == ST_F32 && LEVELS == 2 && 2 * a.g.fs * (long long)sizeof(T) > l2;
+    const int resident = streams && fit > 2 * sms ? 2 * sms : fit;
     const int xs = (a.g.nx + 127) / 128;
     const int ys = (a.g.ny + TY - 1) / TY;
     int H = a.H;
