@@ -358,22 +358,7 @@ cudaError_t launch_tb(const LaunchArgs& a) {
     }
     const int strips = (a.g.nx + kTbLead / 2 + kTbStride - 1) / kTbStride;
     int H = a.H;
-    if (H <= 0) {
-        // rows per item: maximise (output rows / streamed rows) x (fill of the resident warp slots)
-        const long long wslots = (long long)resident * NW;
-        double best = -1.0;
-        for (int h = 8; h <= 512; ++h) {
-            const long long items = (long long)strips * ((a.g.ny + h - 1) / h);
-            const long long rounds = (items + wslots - 1) / wslots;
-            const double fill = (double)items / (double)(rounds * wslots);
-            const double eff = fill * (double)h / (double)(h + 2 * TT);
-            if (eff > best + 1e-9) {
-                best = eff;
-                H = h;
-            }
-            if (h >= a.g.ny) break;
-        }
-    }
+    if (H <= 0) H = march_height(strips, a.g.ny, (long long)resident * NW, 2 * TT, 8, 512);
     const int nitems = strips * ((a.g.ny + H - 1) / H);
     const int blocks_needed = (nitems + NW - 1) / NW;
     const int grid = blocks_needed < resident ? blocks_needed : resident;

@@ -395,6 +395,32 @@ constexpr int march3d_stages() {
 constexpr int kLeanWideRows = 16;
 constexpr size_t kLeanWideRing = 200 * 1024;
 
+// Work split of a 3D launch over `resident` CTAs: *H planes per item, *nitems items, *grid CTAs; or,
+// with `balanced` (and no height asked for), *H = -1: one balanced range of the (y tile, plane)
+// pairs per group of xs CTAs, so every SM gets the same work and a tile's halo planes are read once
+// per range.  The balanced split is for 16-row BF16 tiles, one CTA per SM: nse3d_512 ran 135-136
+// GLUPS against 128 with items of 64 planes; DRAM reads 1.26x the level (384^3 capture), 1.9x when
+// the strips of a row did not share a range.  The FP32 step is bound by DRAM, and there items of
+// planes stay faster (135 against 132 GLUPS with the ranges): neighbouring y tiles' ranges sit at
+// unrelated planes and no longer meet each other's halo rows in L2.
+inline void march3d_split(const Geom& g, int TY, int asked, int resident, bool balanced, int* H, int* nitems, int* grid) {
+    const int xs = (g.nx + 127) / 128;
+    const int ys = (g.ny + TY - 1) / TY;
+    int h0 = asked;
+    if (h0 <= 0 && balanced) {
+        const long long total = (long long)ys * g.nz;     // (y tile, plane) pairs per strip
+        const long long groups = resident >= xs ? resident / xs : 1;
+        *H = -1;
+        *grid = (int)(total < groups ? total : groups) * xs;
+        *nitems = *grid;
+        return;
+    }
+    if (h0 <= 0) h0 = march_height((long long)xs * ys, g.nz, resident, 2, 4, 512);
+    *H = h0;
+    *nitems = xs * ys * ((g.nz + h0 - 1) / h0);
+    *grid = *nitems < resident ? *nitems : resident;
+}
+
 template <int LAT, int PDE, int LEVELS, int ST, int TY, int NSTAGE, int SRC = 0, int LEAN = LEAN_NONE, int SRM = 2>
 cudaError_t launch_march3d_t(const LaunchArgs& a) {
     using T = typename Storage<ST>::T;
@@ -426,41 +452,8 @@ cudaError_t launch_march3d_t(const LaunchArgs& a) {
     // 512^3 174 us with two CTAs per SM against 215 with three; 256^3, in L2, 28.5 against 26.1.
     const bool streams = kAligned && ST == ST_F32 && LEVELS == 2 && 2 * a.g.fs * (long long)sizeof(T) > l2;
     const int resident = streams && fit > 2 * sms ? 2 * sms : fit;
-    const int xs = (a.g.nx + 127) / 128;
-    const int ys = (a.g.ny + TY - 1) / TY;
-    int H = a.H;
-    int nitems = 0, grid = 0;
-    if (H <= 0 && TY == kLeanWideRows && ST == ST_BF16) {
-        // 16-row BF16 tiles, one CTA per SM: each group of xs CTAs streams one balanced range of the
-        // (y tile, plane) pairs, so every SM gets the same work and a tile's halo planes are read
-        // once per range.  nse3d_512: 135-136 GLUPS against 128 with items of 64 planes; DRAM
-        // reads 1.26x the level (384^3 capture), 1.9x when the strips of a row did not share a
-        // range.  The BF16 step is bound by instruction issue; the FP32 step is not, and there
-        // items of planes stay faster (135 against 132 GLUPS with the ranges): neighbouring y
-        // tiles' ranges sit at unrelated planes and no longer meet each other's halo rows in L2.
-        const long long total = (long long)ys * a.g.nz;     // (y tile, plane) pairs per strip
-        const long long groups = resident >= xs ? resident / xs : 1;
-        H = -1;
-        grid = (int)(total < groups ? total : groups) * xs;
-        nitems = grid;
-    } else if (H <= 0) {
-        double best = -1.0;
-        for (int h = 4; h <= 512; ++h) {
-            const long long items = (long long)xs * ys * ((a.g.nz + h - 1) / h);
-            const long long rounds = (items + resident - 1) / resident;
-            const double fill = (double)items / (double)(rounds * resident);
-            const double eff = fill * (double)h / (double)(h + 2);
-            if (eff > best + 1e-9) {
-                best = eff;
-                H = h;
-            }
-            if (h >= a.g.nz) break;
-        }
-    }
-    if (H > 0) {
-        nitems = xs * ys * ((a.g.nz + H - 1) / H);
-        grid = nitems < resident ? nitems : resident;
-    }
+    int H = 0, nitems = 0, grid = 0;
+    march3d_split(a.g, TY, a.H, resident, TY == kLeanWideRows && ST == ST_BF16, &H, &nitems, &grid);
     SrcParam<T, SRC> sa{};
     if constexpr (SRC != 0) {
         sa.s[0] = static_cast<const T*>(a.src[0]);
