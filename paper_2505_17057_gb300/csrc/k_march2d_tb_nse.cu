@@ -1,5 +1,5 @@
 // k_march2d_tb_nse.cu -- temporally blocked 2D He-Luo NSE steps: D2Q9, two levels, the lean
-// streaming form (Coef::nA with streaming momentum), FP32 or BF16 storage.  One launch advances
+// streaming form (Coef::nA with streaming momentum), BF16 storage (FP32: k_march2d_nse.cu).  One launch advances
 // TT time levels and reads / writes the stored level (rho, ux, uy) once.
 //
 // The layout of k_march2d_tb (the scalar blocked kernel) with three fields:
@@ -303,7 +303,7 @@ cudaError_t launch_tbn(const LaunchArgs& a) {
 int march2d_tb_nse_max_depth() { return 3; }
 
 LaunchFn find_march2d_tb_nse(int st, int depth) {
-    if (st == ST_F32) return depth == 2 ? launch_tbn<ST_F32, 2> : depth == 3 ? launch_tbn<ST_F32, 3> : nullptr;
+    if (st == ST_F32) return depth >= 2 ? find_march2d_nse(st, depth) : nullptr;
     if (st == ST_BF16) return depth == 2 ? launch_tbn<ST_BF16, 2> : depth == 3 ? launch_tbn<ST_BF16, 3> : nullptr;
     return nullptr;
 }

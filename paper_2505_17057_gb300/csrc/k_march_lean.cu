@@ -7,6 +7,7 @@ namespace mmfd {
 
 namespace {
 
+// (two-level 2D FP32 solvers with streaming momentum run the class form, see find_march_lean)
 template <int LEVELS, int ST, int LEAN>
 LaunchFn pick2() {
     return launch_march2d_sr<LAT_D2Q9, PDE_NSE, LEVELS, ST, 4, march2d_stages<LAT_D2Q9, PDE_NSE, LEVELS, ST, 4>(), 4,
@@ -27,7 +28,10 @@ LaunchFn pick3(int rows) {
 template <int LEAN>
 LaunchFn pick_dim(int dim, int levels, int st, int rows) {
     if (dim == 2) {
-        if (levels == 2) return st == ST_F32 ? pick2<2, ST_F32, LEAN>() : st == ST_BF16 ? pick2<2, ST_BF16, LEAN>() : nullptr;
+        if constexpr (LEAN == LEAN_GENERAL) {
+            if (levels == 2 && st == ST_F32) return pick2<2, ST_F32, LEAN>();
+        }
+        if (levels == 2) return st == ST_BF16 ? pick2<2, ST_BF16, LEAN>() : nullptr;
         if (levels == 3) return st == ST_F32 ? pick2<3, ST_F32, LEAN>() : st == ST_BF16 ? pick2<3, ST_BF16, LEAN>() : nullptr;
     } else {
         if (levels == 2)
@@ -40,9 +44,17 @@ LaunchFn pick_dim(int dim, int levels, int st, int rows) {
 
 }  // namespace
 
-LaunchFn find_march_lean(int lat, int levels, int st, int lean, int rows) {
+LaunchFn find_march_lean(int lat, int levels, int st, int lean, int nx, int rows) {
     const int dim = lat == LAT_D2Q9 ? 2 : lat == LAT_D3Q19 ? 3 : 0;
     if (dim == 0) return nullptr;
+    if (levels == 2 && lean == LEAN_STREAM && st != ST_BF16) {
+        if (dim == 2) return find_march2d_nse(st, 1);
+        // In 3D the FP32 pushed kernel, with its producer warp, is the faster one where its stores are whole
+        // vectors; class form against pushed, us per step: 512^3 1009 / 974, 384^3 566 / 420, 256^3 154 / 139,
+        // 128^3 25 / 25, but 510 x 512^2 1132 / 2062, 250^3 163 / 301, 131 x 128^2 52 / 86.  Below 128 columns
+        // only the class form marches (kClassMinNx).
+        if (st == ST_F64 || nx < 128 || nx % 4 != 0) return find_march3d_nse(st, rows);
+    }
     if (lean == LEAN_STREAM) return pick_dim<LEAN_STREAM>(dim, levels, st, rows);
     if (lean == LEAN_GENERAL) return pick_dim<LEAN_GENERAL>(dim, levels, st, rows);
     return nullptr;

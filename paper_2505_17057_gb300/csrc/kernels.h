@@ -52,8 +52,10 @@ LaunchFn find_march3d(int lat, int pde, int levels, int st);
 // It reads the level through the same 2-row-box tensor maps as k_march2d.
 LaunchFn find_march2d_tb(int lat, int pde, int levels, int st, int depth);
 int march2d_tb_max_depth(int st);
-// The temporally blocked D2Q9 He-Luo NSE step in the lean streaming form (two levels, FP32 /
-// BF16 storage; depth 2 .. march2d_tb_nse_max_depth()).
+// The D2Q9 He-Luo NSE step in the lean streaming form (two levels), depth steps per launch: FP32 1 .. 3,
+// FP64 1.
+LaunchFn find_march2d_nse(int st, int depth);
+// The temporally blocked one of these, FP32 / BF16 storage (depth 2 .. march2d_tb_nse_max_depth()).
 LaunchFn find_march2d_tb_nse(int st, int depth);
 int march2d_tb_nse_max_depth();
 // The same kernel advancing `depth` Jacobi sweeps of the two-level LCDE theta-scheme per launch
@@ -65,11 +67,15 @@ LaunchFn find_march3d_src(int lat, int pde, int levels, int st, int src);
 // Rows of the x-y tile a 3D march CTA stages per plane (the TMA box is 128+halo x rows+2 x 1).
 int march3d_tile_rows(int pde);
 // The 2D (D2Q9) and 3D (D3Q19) marching kernels in the lean He-Luo NSE form (lean = LEAN_STREAM
-// or LEAN_GENERAL, see Coef::nA; FP32 / BF16 storage, two or three levels; nullptr elsewhere).
+// or LEAN_GENERAL, see Coef::nA; FP32 / BF16 storage, two or three levels; FP64 for the two-level
+// streaming form only; nullptr elsewhere).
 // They take the same tensor maps and launch arguments as find_march2d / find_march3d, except that
 // in 3D `rows` picks the CTA tile: march3d_tile_rows(PDE_NSE) rows at four CTAs per SM, or 16 rows
 // at one CTA per SM (tensor-map boxes of rows + 2 rows either way; 2D ignores it).
-LaunchFn find_march_lean(int lat, int levels, int st, int lean, int rows = 4);
+LaunchFn find_march_lean(int lat, int levels, int st, int lean, int nx, int rows = 4);
+// The D3Q19 He-Luo NSE step in the lean streaming form (two levels; FP32 with rows as for
+// find_march_lean, FP64 with march3d_tile_rows(PDE_NSE) rows).
+LaunchFn find_march3d_nse(int st, int rows);
 // Tile rows a 3D lean solver of this grid runs with: 16 where the grid has enough 16-row tiles to
 // fill the GPU with one CTA per SM, march3d_tile_rows(PDE_NSE) otherwise; force > 0 asks for the
 // 16-row tiles and force < 0 for the narrow ones whatever the grid (for comparisons).

@@ -175,7 +175,7 @@ int mmfd_describe(const mmfd_desc* desc, mmfd_info_t* out) {
     // the step kernel family mmfd_create would pick, as far as it follows from the descriptor
     // alone: the marching kernels from 128 columns (their lean He-Luo variants where the host
     // check accepts the coefficients, FP32 / BF16 storage), the direct kernel below
-    const bool march = r->n[0] >= 128 && !r->theta_on && r->src == 0;
+    const bool march = r->n[0] >= (class_form_3d(*r) ? kClassMinNx : 128) && !r->theta_on && r->src == 0;
     const char* name = "k_direct";
     if (march) {
         const bool lean = r->lean != LEAN_NONE && r->st != ST_F64;

@@ -181,7 +181,7 @@ static int nse_lean(Coef<double>& c, int lat, int dim, int levels) {
         for (int i = 1; i < nin; ++i)
             if (!close(c.oB[p][in[i]] * pair_e(lat, p, in[i]), o[p])) return LEAN_NONE;
     }
-    double eAk[2] = {0.0, 0.0}, qk[2] = {0.0, 0.0};
+    double eAk[2] = {0.0, 0.0}, qk[2] = {0.0, 0.0}, kc[2] = {0.0, 0.0}, oc[2] = {0.0, 0.0};
     bool seen[2] = {false, false};
     for (int p = 0; p < NP; ++p) {
         const int kk = cls[p];
@@ -189,7 +189,9 @@ static int nse_lean(Coef<double>& c, int lat, int dim, int levels) {
             seen[kk] = true;
             eAk[kk] = c.eA[p];
             qk[kk] = q[p];
-        } else if (!close(c.eA[p], eAk[kk]) || !close(q[p], qk[kk])) {
+            kc[kk] = k[p];
+            oc[kk] = o[p];
+        } else if (!close(c.eA[p], eAk[kk]) || !close(q[p], qk[kk]) || !close(k[p], kc[kk]) || !close(o[p], oc[kk])) {
             return LEAN_NONE;
         }
     }
@@ -207,6 +209,13 @@ static int nse_lean(Coef<double>& c, int lat, int dim, int levels) {
         } else if (bm != 0.0 || bp != 0.0) {
             stream = false;   // the level moves momentum but no scalar
         }
+        // (the two-level class forms scale their momentum sums by kappa; the 3D one also takes the
+        // classes' common ratios out, with nA_0 in the denominator)
+        if (nl == 1 && kap[l] == 0.0) stream = false;
+        if (nl == 1 && dim == 3 &&
+            (ap == 0.0 || eAk[0] == 0.0 || !close(qk[0] * eAk[1], qk[1] * eAk[0]) || !close(kc[0] * eAk[1], kc[1] * eAk[0]) ||
+             !close(oc[0] * eAk[1], oc[1] * eAk[0])))
+            stream = false;
     }
     for (int l = 0; l < nl; ++l) {
         const double sE = stream ? c.ap[l] : 1.0, sO = stream ? c.am[l] : 1.0;

@@ -59,4 +59,12 @@ double bytes_per_lu(const Resolved& r);
 // Element size of a storage type.
 inline int storage_bytes(int st) { return st == ST_F64 ? 8 : st == ST_F32 ? 4 : 2; }
 
+// Whether a 3D solver of this problem steps with the kernel in class form (k_march3d_nse),
+// and the fewest columns that kernel takes.
+inline bool class_form_3d(const Resolved& r) {
+    if (r.dim != 3 || r.st == ST_BF16 || r.src || r.theta_on) return false;
+    return r.pde == PDE_NSE && r.lean == LEAN_STREAM && r.levels == 2;
+}
+constexpr int kClassMinNx = 65;
+
 }  // namespace mmfd

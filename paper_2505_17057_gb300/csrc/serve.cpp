@@ -191,7 +191,7 @@ int admit(Server* s, Req* q) {
     q->solo = nullptr;
     const bool large = (long long)q->g.nx * q->g.ny * q->g.nz >= kSoloNodes;
     if (large && q->g.nx >= (q->g.dim == 3 ? 64 : 128)) {
-        LaunchFn fn = find_march_lean(q->r->lat, q->r->levels, q->r->st, q->r->lean);
+        LaunchFn fn = find_march_lean(q->r->lat, q->r->levels, q->r->st, q->r->lean, q->r->n[0]);
         if (!fn)
             fn = q->g.dim == 2 ? find_march2d(q->r->lat, q->r->pde, q->r->levels, q->r->st)
                                : find_march3d(q->r->lat, q->r->pde, q->r->levels, q->r->st);

@@ -487,6 +487,10 @@ static LaunchFn blocked_kernel(const Solver* s, int depth) {
     return find_march2d_tb(s->r.lat, s->r.pde, s->r.levels, s->r.st, depth);
 }
 
+// Narrowest grid the 3D marching kernels take: 128 columns, or kClassMinNx for the kernels in class
+// form, which beat the one-node-per-thread kernel with part of their lanes idle (params.h).
+static int march3d_min_nx(const Resolved& r) { return class_form_3d(r) ? kClassMinNx : 128; }
+
 void solver_use_depth(Solver* s, int depth) {
     LaunchFn fb = nullptr;
     if (depth >= 2 && s->r.theta_on)
@@ -528,10 +532,15 @@ int solver_pick_kernels(Solver* s) {
     // MMFD_FORCE_KERNEL=lean3d_rows16 / lean3d_rows4 picks the tile whatever the grid, for
     // comparisons: both compute every node with the same arithmetic in the same order)
     const int force_rows = !force ? 0 : std::strcmp(force, "lean3d_rows16") == 0 ? 1 : std::strcmp(force, "lean3d_rows4") == 0 ? -1 : 0;
-    const int lean_rows = s->r.dim == 3 ? march3d_lean_tile_rows(s->g.nx, s->g.ny, s->g.nz, force_rows) : 0;
+    const int lean_rows = s->r.dim != 3 ? 0
+                          : s->r.st == ST_F64 ? march3d_tile_rows(PDE_NSE)
+                                              : march3d_lean_tile_rows(s->g.nx, s->g.ny, s->g.nz, force_rows);
     LaunchFn fn_lean =
-        lean != LEAN_NONE ? find_march_lean(s->r.lat, s->r.levels, s->r.st, lean, s->r.dim == 3 ? lean_rows : 4) : nullptr;
-    s->lean = fn_lean ? lean : LEAN_NONE;
+        lean != LEAN_NONE ? find_march_lean(s->r.lat, s->r.levels, s->r.st, lean, s->g.nx, s->r.dim == 3 ? lean_rows : 4) : nullptr;
+    // (FP64 levels, where the class form saves FP64 operations, keep the general name and one step
+    // per launch)
+    s->lean = fn_lean && s->r.st != ST_F64 ? lean : LEAN_NONE;
+    const bool lean3d = fn_lean != nullptr;
     if (s->r.dim == 2 && s->g.nx >= 128 && !want_direct) {
         s->fn = fn_lean ? fn_lean
                 : srcv  ? find_march2d_src(s->r.lat, s->r.pde, s->r.levels, s->r.st, srcv)
@@ -582,7 +591,7 @@ int solver_pick_kernels(Solver* s) {
             return MMFD_OK;
         }
     }
-    if (s->r.dim == 3 && s->g.nx >= 128 && !want_direct) {
+    if (s->r.dim == 3 && s->g.nx >= march3d_min_nx(s->r) && !want_direct) {
         s->fn = fn_lean ? fn_lean
                 : srcv  ? find_march3d_src(s->r.lat, s->r.pde, s->r.levels, s->r.st, srcv)
                         : find_march3d(s->r.lat, s->r.pde, s->r.levels, s->r.st);
@@ -593,12 +602,12 @@ int solver_pick_kernels(Solver* s) {
         if (s->fn) {
             const int es = s->g.es;
             const int boxw = 128 + 2 * (16 / es);
-            s->tile_rows = fn_lean ? lean_rows : march3d_tile_rows(s->r.pde);
+            s->tile_rows = lean3d ? lean_rows : march3d_tile_rows(s->r.pde);
             const int rows = s->tile_rows + 2;
             // the 16-row BF16 kernel streams balanced per-group ranges (k_march3d.cuh): neighbouring
             // y tiles sit at unrelated planes, so L2 promotion would fetch bytes no neighbour reads
             // in time
-            const bool promote = !(fn_lean && s->tile_rows > march3d_tile_rows(s->r.pde) && s->r.st == ST_BF16);
+            const bool promote = !(lean3d && s->tile_rows > march3d_tile_rows(s->r.pde) && s->r.st == ST_BF16);
             for (int b = 0; b < s->nlev && s->fn; ++b)
                 for (int f = 0; f < s->g.nf; ++f) {
                     char* base = static_cast<char*>(s->lev[b]) + (size_t)f * s->g.fs * es;

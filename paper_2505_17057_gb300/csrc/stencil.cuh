@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "mmfd_internal.h"
+#include "pk.cuh"
 
 namespace mmfd {
 
@@ -202,12 +203,6 @@ __device__ __forceinline__ T edot(T ux, T uy, T uz) {
 // multiply-add, none left to the compiler's choice of contraction.  Kernels that evaluate the same
 // node's contributions in different contexts (a value with one use in one kernel, two in another)
 // then round alike.
-__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // Streaming momentum: a contribution sv of pair P in direction SIGN into one output node's
 // accumulators (scalar sv, momentum +-kappa c_a / rho0 times sv).
