@@ -30,6 +30,7 @@ struct LaunchArgs {
     int* err;             // device error flag (bounded waits that ran out)
     const void* src[2];   // source levels t, t - dt (solvers with source terms; else null)
     const void* src_coef; // SrcCoef<double> or SrcCoef<float> matching the storage type
+    const void* cls = nullptr; // NcdeClass<double> or NcdeClass<float> (the NCDE class kernels)
     bool chained = false; // a step of a chain on one stream: launched to overlap its predecessor's end (launch.cuh)
 };
 using LaunchFn = cudaError_t (*)(const LaunchArgs&);
@@ -64,6 +65,10 @@ int march2d_tb_nse_max_depth();
 LaunchFn find_march2d_tb_jacobi(int lat, int st, int depth);
 // The same with source terms in the store epilogue (src as for find_direct_src; LCDE / NCDE).
 LaunchFn find_march3d_src(int lat, int pde, int levels, int st, int src);
+// The 2D (D2Q9) and 3D (D3Q19) NCDE marching kernels in class form (NcdeClass, FP32 / FP64 storage, two or
+// three levels; form = NCLS_GENERAL or NCLS_SHARED; nullptr elsewhere).  They take the tensor maps
+// and launch arguments of find_march2d / find_march3d and LaunchArgs::cls.
+LaunchFn find_march_ncde(int lat, int levels, int st, int form);
 // Rows of the x-y tile a 3D march CTA stages per plane (the TMA box is 128+halo x rows+2 x 1).
 int march3d_tile_rows(int pde);
 // The 2D (D2Q9) and 3D (D3Q19) marching kernels in the lean He-Luo NSE form (lean = LEAN_STREAM

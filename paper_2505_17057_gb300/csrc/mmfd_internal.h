@@ -92,6 +92,19 @@ struct Coef {
 // Lean NSE variants of the marching kernels (Coef::nA): 0 none, 1 streaming momentum, 2 general.
 enum : int { LEAN_NONE = 0, LEAN_STREAM = 1, LEAN_GENERAL = 2 };
 
+// NCDE, class form (host-checked, see ncde_class in params.cpp): where the axes are alike (one speed,
+// one d_0), the even and odd parts of a pair depend only on whether it is an axis (k = 0) or a
+// diagonal pair (k = 1).  Per level l, with a+ and a- folded in,
+//   a+ E_p = eP[l][k] phi + eM[l][k] M2(phi),   a- O_p = oB[l][k] (e_p . B(phi)),
+//   a0 phi + a+ f_0^eq = cP[l] phi + cM[l] M2(phi).
+template <typename T>
+struct NcdeClass {
+    T m2[5], flux[3][4];
+    T eP[2][2], eM[2][2], oB[2][2], cP[2], cM[2];
+};
+// Variants of the NCDE class form: 0 none, 1 general flux, 2 the same flux polynomial on every axis.
+enum : int { NCLS_NONE = 0, NCLS_GENERAL = 1, NCLS_SHARED = 2 };
+
 // Source terms of one step (Eq. (2-1) with F_j = g_j^eq(S, M_1F, 0), Eq. (SourceF)), folded on
 // the host from the central form Eq. (3layerMMFD-2) per level l (0: t, 1: t - dt):
 //   dt [ B_0 S(x) + sum_p omega_p ( b+ (S(x+e_p) - 2 S(x) + S(x-e_p))

@@ -137,6 +137,39 @@ static int coeffs_for(const mmfd_desc& d, const double* explicit_a, const double
     return MMFD_OK;
 }
 
+// NCDE class form (NcdeClass): available on D2Q9 / D3Q19 where every axis pair has the same folded
+// coefficients and every diagonal pair too (one speed and one d_0 on every axis).  Fills `o` and
+// returns NCLS_SHARED when the axes also have the same flux polynomial, NCLS_GENERAL when not.
+static int ncde_class(const Coef<double>& c, int lat, int dim, int levels, NcdeClass<double>& o) {
+    auto close = [](double x, double y) { return x == y || std::fabs(x - y) <= 1e-13 * (std::fabs(x) + std::fabs(y)); };
+    if (lat != LAT_D2Q9 && lat != LAT_D3Q19) return NCLS_NONE;
+    const int DG = dim;   // first diagonal pair
+    for (int p = 0; p < lat_npair(lat); ++p) {
+        const int first = p < dim ? 0 : DG;
+        if (!close(c.ePhi[p], c.ePhi[first]) || !close(c.eM2[p], c.eM2[first])) return NCLS_NONE;
+        for (int a = 0; a < dim; ++a)
+            if (pair_e(lat, p, a) != 0 && !close(c.oB[p][a] * pair_e(lat, p, a), c.oB[first][0])) return NCLS_NONE;
+    }
+    for (int k = 0; k < 5; ++k) o.m2[k] = c.m2[k];
+    for (int a = 0; a < 3; ++a)
+        for (int k = 0; k < 4; ++k) o.flux[a][k] = a < dim ? c.flux[a][k] : 0.0;
+    for (int l = 0; l < 2; ++l) {
+        const bool in = l < levels - 1;
+        for (int k = 0; k < 2; ++k) {
+            const int p = k == 0 ? 0 : DG;
+            o.eP[l][k] = in ? c.ap[l] * c.ePhi[p] : 0.0;
+            o.eM[l][k] = in ? c.ap[l] * c.eM2[p] : 0.0;
+            o.oB[l][k] = in ? c.am[l] * c.oB[p][0] : 0.0;
+        }
+        o.cP[l] = in ? c.a0[l] + c.ap[l] * c.rPhi : 0.0;
+        o.cM[l] = in ? c.ap[l] * c.rM2 : 0.0;
+    }
+    for (int a = 1; a < dim; ++a)
+        for (int k = 0; k < 4; ++k)
+            if (c.flux[a][k] != c.flux[0][k]) return NCLS_GENERAL;
+    return NCLS_SHARED;
+}
+
 // Lean He-Luo form (Coef::nA): whether the folded EDF coefficients of every pair p have the shape
 //   E_p = eA_k rho + q_k |u|^2 + k_p (e_p . u)^2,   O_p = o_p (e_p . u)
 // with eA_k, q_k shared by the axis pairs (k = 0) and by the diagonal pairs (k = 1), and an equal
@@ -491,6 +524,16 @@ int resolve(const mmfd_desc& d_in, Resolved& r, std::string* msg) {
     }
     for (int f = 0; f < 4; ++f) c.ref[f] = r.ref[f];
     r.lean = (d.pde == PDE_NSE && !axis) ? nse_lean(c, d.lattice, dim, d.levels) : LEAN_NONE;
+
+    r.ncls = NCLS_NONE;
+    std::memset(&r.ncd, 0, sizeof(r.ncd));
+    if (d.pde == PDE_NCDE) r.ncls = ncde_class(c, d.lattice, dim, d.levels, r.ncd);
+    {
+        const double* src = reinterpret_cast<const double*>(&r.ncd);
+        float* dst = reinterpret_cast<float*>(&r.ncf);
+        static_assert(sizeof(NcdeClass<double>) == 2 * sizeof(NcdeClass<float>), "NcdeClass layout");
+        for (size_t i = 0; i < sizeof(NcdeClass<double>) / sizeof(double); ++i) dst[i] = (float)src[i];
+    }
 
     // float copy
     {

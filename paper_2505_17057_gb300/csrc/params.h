@@ -22,6 +22,9 @@ struct Resolved {
     double max_lambda;
     Coef<double> cd;
     Coef<float> cf;
+    int ncls;           // NCLS_*: NCDE class form available to the marching kernels
+    NcdeClass<double> ncd;
+    NcdeClass<float> ncf;
     int lean;           // LEAN_*: lean He-Luo form available to the marching kernels
     int src;            // MMFD_SRC_* (0: none)
     int nsrc;           // source fields per level (S, then M_1F components)
@@ -59,11 +62,11 @@ double bytes_per_lu(const Resolved& r);
 // Element size of a storage type.
 inline int storage_bytes(int st) { return st == ST_F64 ? 8 : st == ST_F32 ? 4 : 2; }
 
-// Whether a 3D solver of this problem steps with the kernel in class form (k_march3d_nse),
-// and the fewest columns that kernel takes.
+// Whether a 3D solver of this problem steps with a kernel in class form (k_march3d_nse, k_march3d_ncde),
+// and the fewest columns those kernels take.
 inline bool class_form_3d(const Resolved& r) {
     if (r.dim != 3 || r.st == ST_BF16 || r.src || r.theta_on) return false;
-    return r.pde == PDE_NSE && r.lean == LEAN_STREAM && r.levels == 2;
+    return (r.pde == PDE_NSE && r.lean == LEAN_STREAM && r.levels == 2) || (r.pde == PDE_NCDE && r.ncls != NCLS_NONE);
 }
 constexpr int kClassMinNx = 65;
 

@@ -214,6 +214,7 @@ void solver_launch_args(Solver* s, LaunchArgs& a) {
     a.err = s->d_flag;
     a.maps = nullptr;
     a.chained = s->chained;
+    a.cls = s->r.st == ST_F64 ? static_cast<const void*>(&s->r.ncd) : static_cast<const void*>(&s->r.ncf);
     a.src[0] = s->r.src ? s->srcbuf[s->src_i0] : nullptr;
     a.src[1] = s->r.src ? s->srcbuf[s->src_i1] : nullptr;
     a.src_coef = s->r.st == ST_F64 ? static_cast<const void*>(&s->r.sd) : static_cast<const void*>(&s->r.sf);
@@ -540,7 +541,11 @@ int solver_pick_kernels(Solver* s) {
     // (FP64 levels, where the class form saves FP64 operations, keep the general name and one step
     // per launch)
     s->lean = fn_lean && s->r.st != ST_F64 ? lean : LEAN_NONE;
-    const bool lean3d = fn_lean != nullptr;
+    // the NCDE class form where the axes are alike (FP32 / FP64 storage)
+    const LaunchFn fn_ncde =
+        s->r.pde == PDE_NCDE && !want_generic && !srcv ? find_march_ncde(s->r.lat, s->r.levels, s->r.st, s->r.ncls) : nullptr;
+    if (!fn_lean) fn_lean = fn_ncde;
+    const bool lean3d = fn_lean && !fn_ncde;
     if (s->r.dim == 2 && s->g.nx >= 128 && !want_direct) {
         s->fn = fn_lean ? fn_lean
                 : srcv  ? find_march2d_src(s->r.lat, s->r.pde, s->r.levels, s->r.st, srcv)
