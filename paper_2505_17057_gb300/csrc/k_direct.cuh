@@ -44,25 +44,20 @@ __device__ __forceinline__ T source_level(const Geom& g, const T* __restrict__ s
     return acc;
 }
 
-// The update of one node (x, y, z): reads levels t (in0) and t - dt (in1) in the ghosted
-// layout, writes level t + dt (out) and its periodic ghost images.  Shared by the one-solve
-// kernel below and the batched multi-request kernel, so a request computes the same bits
-// alone and inside a batch.
-// With SRC != 0 the source terms of `sa` are added before the store.
+// The updated fields of the node at offset c0 of levels t (in0) and t - dt (in1) in the layout g.
+// Shared by the one-solve kernel below, the batched multi-request kernel and the cluster kernel, so
+// a solve computes the same bits in each.  With SRC != 0 the source terms of `sa` are added.
 template <int LAT, int PDE, int LEVELS, int ST, int SRC = 0>
-__device__ __forceinline__ void direct_node(const Geom& g, const void* __restrict__ in0v,
-                                            const void* __restrict__ in1v, void* __restrict__ outv,
-                                            const Coef<typename Storage<ST>::T>& cf, const StepExtra& ex,
-                                            int x, int y, int z,
-                                            const SrcArgs<typename Storage<ST>::T>* sa = nullptr) {
+__device__ __forceinline__ void direct_value(const Geom& g, const void* in0v, const void* in1v,
+                                             const Coef<typename Storage<ST>::T>& cf, long long c0,
+                                             typename Storage<ST>::T (&acc)[pde_nf(PDE, LAT)],
+                                             const SrcArgs<typename Storage<ST>::T>* sa = nullptr) {
     using Tr = Storage<ST>;
     using S = typename Tr::S;
     using T = typename Tr::T;
     constexpr int D = lat_dim(LAT);
     constexpr int NP = lat_npair(LAT);
     constexpr int NF = pde_nf(PDE, LAT);
-    const long long c0 = g.at(x, y, z);
-    T acc[NF];
 #pragma unroll
     for (int i = 0; i < NF; ++i) acc[i] = T(0);
 
@@ -118,6 +113,22 @@ __device__ __forceinline__ void direct_node(const Geom& g, const void* __restric
 #pragma unroll
         for (int l = 0; l < LEVELS - 1; ++l) acc[0] += source_level<LAT, SRC, T>(g, sa->s[l], sa->w, l, c0);
     }
+}
+
+// The update of one node (x, y, z): reads levels t (in0) and t - dt (in1) in the ghosted
+// layout, writes level t + dt (out) and its periodic ghost images.
+template <int LAT, int PDE, int LEVELS, int ST, int SRC = 0>
+__device__ __forceinline__ void direct_node(const Geom& g, const void* __restrict__ in0v,
+                                            const void* __restrict__ in1v, void* __restrict__ outv,
+                                            const Coef<typename Storage<ST>::T>& cf, const StepExtra& ex,
+                                            int x, int y, int z,
+                                            const SrcArgs<typename Storage<ST>::T>* sa = nullptr) {
+    using S = typename Storage<ST>::S;
+    using T = typename Storage<ST>::T;
+    constexpr int D = lat_dim(LAT);
+    constexpr int NF = pde_nf(PDE, LAT);
+    T acc[NF];
+    direct_value<LAT, PDE, LEVELS, ST, SRC>(g, in0v, in1v, cf, g.at(x, y, z), acc, sa);
     S* out = static_cast<S*>(outv);
     const long long node = ((long long)z * g.ny + y) * g.nx + x;
 #pragma unroll

@@ -35,6 +35,23 @@ struct LaunchArgs {
 };
 using LaunchFn = cudaError_t (*)(const LaunchArgs&);
 
+// A launch advancing nsteps steps of a small 2D solve in one thread-block cluster: the level buffers
+// lev[0 .. levels), level t in lev[cur]; afterwards level t + nsteps dt is in the buffer that as many
+// single steps would leave it in, level t - dt (three levels) in that one's predecessor, and the
+// other buffer is as it was.  cudaErrorNotSupported if the device does not schedule the cluster.
+struct ClusterArgs {
+    Geom g;
+    void* lev[3];
+    int cur;
+    const void* coef;
+    StepExtra ex;          // step: that of the first new level
+    int nsteps;
+    cudaStream_t stream;
+};
+using ClusterFn = cudaError_t (*)(const ClusterArgs&);
+// The cluster kernel of a solve, or null where one launch per step is the better choice.
+ClusterFn find_cluster(int lat, int pde, int levels, int st, const Geom& g);
+
 // One node per thread, neighbours read straight from the ghosted layout (any shape).
 LaunchFn find_direct(int lat, int pde, int levels, int st);
 // The same with source terms: src 1 (a source S, M_1F = 0 or S u folded) or 2 (S and M_1F fields).

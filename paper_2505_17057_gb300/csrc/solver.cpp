@@ -280,6 +280,27 @@ int solver_step(Solver* s, long long nsteps) {
         return MMFD_OK;
     }
     long long done = 0;
+    while (s->fn_cluster && nsteps - done >= 2) {
+        ClusterArgs c;
+        c.g = s->g;
+        for (int i = 0; i < 3; ++i) c.lev[i] = s->lev[i];
+        c.cur = s->cur;
+        c.coef = s->coef();
+        c.ex.seed = s->desc.seed;
+        c.ex.step = s->steps_done + 1;
+        c.ex.sr = (s->r.st == ST_BF16 && (s->desc.flags & MMFD_FLAG_STOCHASTIC_ROUND)) ? 1 : 0;
+        c.nsteps = (int)(nsteps - done < 100000 ? nsteps - done : 100000);
+        c.stream = s->stream;
+        cudaError_t e = s->fn_cluster(c);
+        if (e == cudaErrorNotSupported) {
+            s->fn_cluster = nullptr;
+            break;
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "cluster step kernel");
+        s->cur = (int)((s->cur + c.nsteps) % s->nlev);
+        s->steps_done += c.nsteps;
+        done += c.nsteps;
+    }
     while (done < nsteps) {
         const long long left = nsteps - done;
         const bool blocked = s->fn_block && s->depth > 1 && left >= s->depth;
@@ -513,6 +534,7 @@ void solver_use_depth(Solver* s, int depth) {
 
 int solver_pick_kernels(Solver* s) {
     s->fn_block = nullptr;
+    s->fn_cluster = nullptr;
     s->depth = 1;
     s->max_depth = 1;
     s->variant = 0;
@@ -635,6 +657,8 @@ int solver_pick_kernels(Solver* s) {
     s->fn = srcv ? find_direct_src(s->r.lat, s->r.pde, s->r.levels, s->r.st, srcv)
                  : find_direct(s->r.lat, s->r.pde, s->r.levels, s->r.st);
     s->kernel_name = srcv ? "k_direct_src" : "k_direct";
+    if (!srcv && !s->r.theta_on && !s->r.dirichlet && !want_direct)
+        s->fn_cluster = find_cluster(s->r.lat, s->r.pde, s->r.levels, s->r.st, s->g);
     if (s->r.theta_on) s->fn_rhs = find_direct(s->r.lat, s->r.pde, s->r.levels, s->r.st);
     if (!s->fn || (s->r.theta_on && !s->fn_rhs))
         return set_error(MMFD_ERR_UNSUPPORTED, "no kernel for this lattice/PDE/levels/storage");

@@ -30,6 +30,7 @@ struct Solver {
     int depth = 1;                               // steps fused per launch
     int max_depth = 1;                           // deepest blocking this solver's ghosts allow
     LaunchFn fn = nullptr;                       // single-step kernel
+    ClusterFn fn_cluster = nullptr;              // all steps of a call in one launch (small grids)
     LaunchFn fn_block = nullptr;                 // temporally blocked kernel (depth > 1)
     int variant = 0;
     const char* kernel_name = "k_direct";
