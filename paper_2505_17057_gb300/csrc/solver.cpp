@@ -247,33 +247,41 @@ int solver_step(Solver* s, long long nsteps) {
         const bool f64 = s->r.st == ST_F64;
         for (long long n = 0; n < nsteps; ++n) {
             LaunchArgs a;
+            int left = s->r.sweeps;
+            if (s->fn_block && s->depth > 1) {
+                // fused kernels: one pass for rhs / d and the first sweep, then `depth` sweeps per launch
+                // (fewer, with the launcher's own work-item height, for the remainder)
+                solver_launch_args(s, a);
+                a.coef2 = f64 ? static_cast<const void*>(&s->r.thq_d) : static_cast<const void*>(&s->r.thq_f);
+                a.src_coef = f64 ? static_cast<const void*>(&s->r.th1_d) : static_cast<const void*>(&s->r.th1_f);
+                a.H = 0;
+                cudaError_t e = s->fn_rhs(a);
+                if (e != cudaSuccess) return cuda_fail(e, "theta-scheme first pass kernel");
+                s->cur = s->next();
+                for (--left; left > 0;) {
+                    solver_launch_args(s, a);
+                    const int did = left < s->depth ? left : s->depth;
+                    const LaunchFn f = did == s->depth ? s->fn_block : find_march2d_theta(s->r.lat, s->r.st, did);
+                    if (did != s->depth) a.H = 0;
+                    e = f(a);
+                    if (e != cudaSuccess) return cuda_fail(e, "theta-scheme sweep kernel");
+                    s->cur = s->next();
+                    left -= did;
+                }
+                s->steps_done += 1;
+                continue;
+            }
             solver_launch_args(s, a);
             a.out = s->rhs;
             a.coef = f64 ? static_cast<const void*>(&s->r.thr_d) : static_cast<const void*>(&s->r.thr_f);
             a.src[0] = a.src[1] = nullptr;
             cudaError_t e = s->fn_rhs(a);
             if (e != cudaSuccess) return cuda_fail(e, "theta-scheme right-hand side kernel");
-            // sweeps fused `depth` per launch by the blocked kernel (a shallower blocked launch,
-            // with the launcher's own work-item height, or a single sweep for the remainder)
-            int left = s->r.sweeps;
-            while (left > 0) {
+            for (; left > 0; --left) {
                 solver_launch_args(s, a);
-                LaunchFn f = s->fn;
-                int did = 1;
-                if (s->fn_block && s->depth > 1 && left >= 2) {
-                    did = left >= s->depth ? s->depth : left;
-                    f = did == s->depth ? s->fn_block : find_march2d_tb_jacobi(s->r.lat, s->r.st, did);
-                    if (did != s->depth) a.H = 0;
-                    if (!f) {
-                        f = s->fn;
-                        did = 1;
-                        a.H = s->H;
-                    }
-                }
-                e = f(a);
+                e = s->fn(a);
                 if (e != cudaSuccess) return cuda_fail(e, "theta-scheme sweep kernel");
                 s->cur = s->next();
-                left -= did;
             }
             s->steps_done += 1;
         }
@@ -516,9 +524,11 @@ static int march3d_min_nx(const Resolved& r) { return class_form_3d(r) ? kClassM
 void solver_use_depth(Solver* s, int depth) {
     LaunchFn fb = nullptr;
     if (depth >= 2 && s->r.theta_on)
-        fb = s->r.dim == 2 ? find_march2d_tb_jacobi(s->r.lat, s->r.st, depth) : nullptr;
+        fb = s->r.dim == 2 ? find_march2d_theta(s->r.lat, s->r.st, depth) : nullptr;
     else if (depth >= 2)
         fb = blocked_kernel(s, depth);
+    if (s->r.theta_on && s->r.dim == 2 && s->use_tma)
+        s->fn_rhs = fb ? find_march2d_theta(s->r.lat, s->r.st, 0) : find_march2d(s->r.lat, s->r.pde, s->r.levels, s->r.st);
     if (fb) {
         s->fn_block = fb;
         s->depth = depth;
@@ -601,7 +611,7 @@ int solver_pick_kernels(Solver* s) {
             if (s->r.pde == PDE_NSE && maxd > march2d_tb_nse_max_depth()) maxd = march2d_tb_nse_max_depth();
             while (maxd >= 2 && s->g.ny < 2 * maxd) --maxd;
             if (s->r.theta_on && s->desc.temporal_depth != 1 && maxd >= 2 &&
-                find_march2d_tb_jacobi(s->r.lat, s->r.st, 2)) {
+                find_march2d_theta(s->r.lat, s->r.st, 2)) {
                 // theta-scheme: Jacobi sweeps fused per launch
                 s->max_depth = maxd;
                 int want = s->desc.temporal_depth == 0 ? maxd : s->desc.temporal_depth;
