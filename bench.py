@@ -724,32 +724,31 @@ def run_ours(args):
         alg_bytes = bytes_per_lu * nodes
         effective = bytes_per_lu * nodes * depth / avg_launch_s / 1e9
         kernel_name = info.kernel.decode()
-        # theta-scheme: one step is the right-hand side plus info.sweeps Jacobi sweeps, fused jd
-        # per launch; its events, bytes and traffic are those of the whole step.  Compulsory bytes:
-        # the right-hand side reads the level and writes rhs, each sweep launch reads the iterate
-        # and rhs and writes the next iterate; the effective figure counts every sweep as unfused.
+        # theta-scheme: one step is the right-hand side plus info.sweeps Jacobi sweeps; its events,
+        # bytes and traffic are those of the whole step.  Fused (jd > 1), the right-hand side's pass
+        # also writes the first sweep's result and the others run jd per launch.  Compulsory bytes:
+        # the right-hand side reads the level and writes rhs (fused: and the iterate), each sweep
+        # launch reads the iterate and rhs and writes the next iterate; the effective figure counts
+        # every sweep as unfused.
         theta = info.sweeps > 0
         jd = max(1, info.temporal_depth)
-        sweep_launches = info.sweeps // jd + (1 if info.sweeps % jd else 0)
+        left = info.sweeps - 1 if jd > 1 else info.sweeps
+        sweep_launches = -(-left // jd)
         launches_per_step = (1 + sweep_launches) if theta else 1
         theta_launches = None
         if theta:
-            # what one step launches: the right-hand side, then the sweeps (fused jd per launch; a
-            # remainder of one runs on the single-sweep kernel, a longer one on a shallower fused launch)
-            full, rem = divmod(info.sweeps, jd)
-            single = kernel_name.replace("_tb", "_src") if kernel_name.endswith("_tb") else kernel_name
-            parts = [kernel_name.replace("_tb", "").replace("_src", "") + " (right-hand side)"]
+            # what one step launches: the right-hand side, then the sweeps (fused jd per launch, a
+            # remainder on a shallower fused launch)
+            full, rem = divmod(left, jd)
             if jd > 1:
-                parts.append(f"{full} x {kernel_name} ({jd} sweeps each)")
-                if rem == 1:
-                    parts.append(f"1 x {single}")
-                elif rem > 1:
-                    parts.append(f"1 x {kernel_name} ({rem} sweeps)")
+                parts = ["k_theta (right-hand side and first sweep)", f"{full} x k_theta ({jd} sweeps each)"]
+                if rem:
+                    parts.append(f"1 x k_theta ({rem} sweeps)")
             else:
-                parts.append(f"{info.sweeps} x {kernel_name}")
+                parts = [kernel_name.replace("_src", "") + " (right-hand side)", f"{info.sweeps} x {kernel_name}"]
             theta_launches = " + ".join(parts)
             es = {"fp32": 4, "fp64": 8}[args.storage]
-            alg_bytes = es * (2 + 3 * sweep_launches) * nodes
+            alg_bytes = es * ((3 if jd > 1 else 2) + 3 * sweep_launches) * nodes
             effective = bytes_per_lu * nodes / avg_launch_s / 1e9
         achieved = alg_bytes / avg_launch_s / 1e9
         traffic = traffic_from_profile("k_march2d_theta" if theta else kernel_name, args.workload,

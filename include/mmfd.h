@@ -119,9 +119,11 @@ typedef void (*mmfd_free_fn)(void* ptr, void* ctx);
  *                        the depth in use.  mmfd_step(n) runs n / T blocked launches and the
  *                        remaining n % T steps unblocked.  With BF16 storage a blocked solver
  *                        rounds the state to BF16 once per T steps (the intermediate levels
- *                        stay in FP32).  For a theta-scheme solver (MMFD_FLAG_THETA) the depth
+ *                        stay in FP32).  Small 2D grids on the direct kernel run all steps of
+ *                        a call in one launch, with the same results.  For a theta-scheme solver (MMFD_FLAG_THETA) the depth
  *                        counts Jacobi sweeps fused per launch instead (2D grids with nx >= 128,
- *                        up to 2 for FP64 and 4 for FP32); every mmfd_step is one time step.
+ *                        up to 2 for FP64 and 4 for FP32; the first sweep comes with the
+ *                        right-hand side's pass); every mmfd_step is one time step.
  *  seed                  BF16 stochastic-rounding seed.
  *  stream                cudaStream_t (NULL = legacy default stream).
  *  alloc/free_fn/ctx     device allocator for the level buffers (NULL = cudaMalloc/cudaFree).
@@ -389,7 +391,8 @@ int mmfd_autotune(mmfd_solver* s, const char* cache_path, mmfd_tune_info* out);
 
 /* Resolve a descriptor's constants without touching the GPU (info filled as by create; kernel
  * names the step kernel family create would pick for a periodic explicit solver: the marching
- * kernels from 128 columns -- k_march2d / k_march3d, or their lean He-Luo NSE variants *_nse_s
+ * kernels from 128 columns (3D two-level streaming NSE, and NCDE with alike axes, FP32 / FP64: from 65)
+ * -- k_march2d / k_march3d, or their lean He-Luo NSE variants *_nse_s
  * (streaming momentum) and *_nse_g (general momentum) for FP32 / BF16 storage with one speed on
  * every axis on D2Q9, or on D3Q19 with d_0 = 1/3 -- and k_direct otherwise). */
 int mmfd_describe(const mmfd_desc* desc, mmfd_info_t* out);
