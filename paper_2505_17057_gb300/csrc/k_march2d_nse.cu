@@ -17,7 +17,7 @@
 // - Columns within TT of the x edges are read from the ghost columns, which every writer keeps
 //   current to the ghost depth.
 //
-// Bound by FP32 issue when blocked (42.7 instructions per node and step, the FMA pipe 65% busy), by DRAM with
+// Bound by FP32 issue when blocked (46 instructions per node and step, the FMA pipe 64% busy), by DRAM with
 // one step per launch.  4096^2 FP32: three steps per launch 35.2 us per step (the pushed form 39.1), one
 // 75 us (77); FP64, bound by the FP64 rate, 1000 x 800 108 us (193).
 // FP32 and FP64 storage; BF16 levels keep the pushed form and its rounding (k_march2d_tb_nse,
