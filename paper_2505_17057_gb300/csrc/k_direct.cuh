@@ -20,24 +20,22 @@ __device__ __forceinline__ void static_for(F&& f) {
 }
 
 // Source term of level l at node c0 (weights folded on the host, see SrcCoef): SRC 1 reads S
-// only (M_1F = 0 or S u), SRC 2 also the M_1F components.  Source levels are read-only for
-// the whole launch, so they go through the read-only data path.
+// only (M_1F = 0 or S u), SRC 2 also the M_1F components.
 template <int LAT, int SRC, typename T>
-__device__ __forceinline__ T source_level(const Geom& g, const T* __restrict__ src, const SrcCoef<T>& w, int l,
-                                          long long c0) {
+__device__ __forceinline__ T source_level(const Geom& g, const T* src, const SrcCoef<T>& w, int l, long long c0) {
     constexpr int NP = lat_npair(LAT);
     constexpr int D = lat_dim(LAT);
-    T acc = w.W0[l] * __ldg(src + c0);
+    T acc = w.W0[l] * src[c0];
     static_for<0, NP>([&](auto pc) {
         constexpr int P = decltype(pc)::value;
         const long long off = pair_offset<LAT>(g, P);
-        acc += w.Wp[l][P] * __ldg(src + c0 + off) + w.Wm[l][P] * __ldg(src + c0 - off);
+        acc += w.Wp[l][P] * src[c0 + off] + w.Wm[l][P] * src[c0 - off];
         if constexpr (SRC == 2) {
 #pragma unroll
             for (int a = 0; a < D; ++a)
                 if (pair_e(LAT, P, a) != 0) {
                     const T* m = src + (long long)(1 + a) * g.fs;
-                    acc += w.M[l][P][a] * (__ldg(m + c0 + off) - __ldg(m + c0 - off));
+                    acc += w.M[l][P][a] * (m[c0 + off] - m[c0 - off]);
                 }
         }
     });
@@ -118,8 +116,7 @@ __device__ __forceinline__ void direct_value(const Geom& g, const void* in0v, co
 // The update of one node (x, y, z): reads levels t (in0) and t - dt (in1) in the ghosted
 // layout, writes level t + dt (out) and its periodic ghost images.
 template <int LAT, int PDE, int LEVELS, int ST, int SRC = 0>
-__device__ __forceinline__ void direct_node(const Geom& g, const void* __restrict__ in0v,
-                                            const void* __restrict__ in1v, void* __restrict__ outv,
+__device__ __forceinline__ void direct_node(const Geom& g, const void* in0v, const void* in1v, void* outv,
                                             const Coef<typename Storage<ST>::T>& cf, const StepExtra& ex,
                                             int x, int y, int z,
                                             const SrcArgs<typename Storage<ST>::T>* sa = nullptr) {
@@ -139,8 +136,7 @@ __device__ __forceinline__ void direct_node(const Geom& g, const void* __restric
 }
 
 template <int LAT, int PDE, int LEVELS, int ST>
-__global__ void __launch_bounds__(256) k_direct(Geom g, const void* __restrict__ in0v,
-                                                const void* __restrict__ in1v, void* __restrict__ outv,
+__global__ void __launch_bounds__(256) k_direct(Geom g, const void* in0v, const void* in1v, void* outv,
                                                 Coef<typename Storage<ST>::T> cf, StepExtra ex) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -160,8 +156,7 @@ cudaError_t launch_direct(const LaunchArgs& a) {
 }
 
 template <int LAT, int PDE, int LEVELS, int ST, int SRC>
-__global__ void __launch_bounds__(256) k_direct_src(Geom g, const void* __restrict__ in0v,
-                                                    const void* __restrict__ in1v, void* __restrict__ outv,
+__global__ void __launch_bounds__(256) k_direct_src(Geom g, const void* in0v, const void* in1v, void* outv,
                                                     Coef<typename Storage<ST>::T> cf, StepExtra ex,
                                                     const __grid_constant__ SrcArgs<typename Storage<ST>::T> sa) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;

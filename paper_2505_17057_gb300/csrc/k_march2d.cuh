@@ -409,21 +409,21 @@ __device__ __forceinline__ void lean_push_node2d(const Coef<T>& cf, int l, const
 // load for the lane's own four (16-byte aligned in the source layout) and two scalars; columns
 // beyond the right ghost column are not read (lanes past nx only feed nodes that are not stored).
 template <typename T>
-__device__ __forceinline__ void ld_src6(const T* __restrict__ row, int xb, int nx, T (&v)[6]) {
+__device__ __forceinline__ void ld_src6(const T* row, int xb, int nx, T (&v)[6]) {
     if (xb + 3 < nx) {
         if constexpr (sizeof(T) == 4) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(row + xb));
+            const float4 q = *reinterpret_cast<const float4*>(row + xb);
             v[1] = q.x; v[2] = q.y; v[3] = q.z; v[4] = q.w;
         } else {
-            const double2 a = __ldg(reinterpret_cast<const double2*>(row + xb));
-            const double2 b = __ldg(reinterpret_cast<const double2*>(row + xb + 2));
+            const double2 a = *reinterpret_cast<const double2*>(row + xb);
+            const double2 b = *reinterpret_cast<const double2*>(row + xb + 2);
             v[1] = a.x; v[2] = a.y; v[3] = b.x; v[4] = b.y;
         }
-        v[0] = __ldg(row + xb - 1);
-        v[5] = __ldg(row + xb + 4);
+        v[0] = row[xb - 1];
+        v[5] = row[xb + 4];
     } else {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) v[c] = xb - 1 + c <= nx ? __ldg(row + xb - 1 + c) : T(0);
+        for (int c = 0; c < 6; ++c) v[c] = xb - 1 + c <= nx ? row[xb - 1 + c] : T(0);
     }
 }
 
@@ -494,8 +494,8 @@ __device__ __forceinline__ void source_quad(const Geom& g, const SrcArgs<T>& sa,
 template <int LAT, int PDE, int LEVELS, int ST, int NW, int NSTAGE, int LN, int RPS, int SRC = 0, int LEAN = LEAN_NONE,
           int SRM = 2>
 __global__ void __launch_bounds__(NW * 32) k_march2d(const __grid_constant__ TmapSet maps, Geom g,
-                                                     void* __restrict__ outv, Coef<typename Storage<ST>::T> cf,
-                                                     StepExtra ex, int H, int nitems, int* __restrict__ err,
+                                                     void* outv, Coef<typename Storage<ST>::T> cf,
+                                                     StepExtra ex, int H, int nitems, int* err,
                                                      const __grid_constant__ SrcParam<typename Storage<ST>::T, SRC> sa) {
     using Tr = Storage<ST>;
     using S = typename Tr::S;

@@ -35,8 +35,8 @@ constexpr int kTbnLead = 8;       // lane 0's first column lies kTbnLead columns
 
 template <int ST, int TT, int NW, int NSTAGE>
 __global__ void __launch_bounds__(NW * 32) k_march2d_nse(const __grid_constant__ TmapSet maps, Geom g,
-                                                            void* __restrict__ outv,
-                                                            ClassCoef<typename Storage<ST>::T> cc, int H, int nitems, int* __restrict__ err) {
+                                                            void* outv, ClassCoef<typename Storage<ST>::T> cc, int H,
+                                                            int nitems, int* err) {
     using Tr = Storage<ST>;
     using S = typename Tr::S;
     using T = typename Tr::T;

@@ -96,8 +96,8 @@ constexpr int tb_min_ctas(int pde, int st, int tt) {
 
 template <int LAT, int PDE, int ST, int TT, int NW, int NSTAGE>
 __global__ void __launch_bounds__(NW * 32, tb_min_ctas(PDE, ST, TT)) k_march2d_tb(const __grid_constant__ TmapSet maps, Geom g,
-                                                        void* __restrict__ outv, Coef<typename Storage<ST>::T> cf,
-                                                        StepExtra ex, int H, int nitems, int* __restrict__ err) {
+                                                        void* outv, Coef<typename Storage<ST>::T> cf,
+                                                        StepExtra ex, int H, int nitems, int* err) {
     using Tr = Storage<ST>;
     using S = typename Tr::S;
     using T = typename Tr::T;

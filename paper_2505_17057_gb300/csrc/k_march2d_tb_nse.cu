@@ -80,8 +80,8 @@ __device__ __forceinline__ void tb_push_row(const Coef<T>& cf, const T (&raw)[LN
 
 template <int ST, int TT, int NW, int NSTAGE, int SRM>
 __global__ void __launch_bounds__(NW * 32) k_march2d_tb_nse(const __grid_constant__ TmapSet maps, Geom g,
-                                                            void* __restrict__ outv, Coef<typename Storage<ST>::T> cf,
-                                                            StepExtra ex, int H, int nitems, int* __restrict__ err) {
+                                                            void* outv, Coef<typename Storage<ST>::T> cf,
+                                                            StepExtra ex, int H, int nitems, int* err) {
     using Tr = Storage<ST>;
     using S = typename Tr::S;
     using T = typename Tr::T;

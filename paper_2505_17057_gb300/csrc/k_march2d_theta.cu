@@ -69,9 +69,9 @@ struct RowBox {
 // else the sweeps (rhs is read, B is J).
 template <int LAT, int ST, int TT, bool FIRST, int NW>
 __global__ void __launch_bounds__(NW * 32, ST == ST_F32 ? 4 : 1)
-    k_theta(const __grid_constant__ TmapSet maps, Geom g, typename Storage<ST>::S* __restrict__ out,
-            typename Storage<ST>::S* __restrict__ rhs, const __grid_constant__ Stencil<typename Storage<ST>::T> A,
-            const __grid_constant__ Stencil<typename Storage<ST>::T> B, int H, int nitems, int* __restrict__ err) {
+    k_theta(const __grid_constant__ TmapSet maps, Geom g, typename Storage<ST>::S* out,
+            typename Storage<ST>::S* rhs, const __grid_constant__ Stencil<typename Storage<ST>::T> A,
+            const __grid_constant__ Stencil<typename Storage<ST>::T> B, int H, int nitems, int* err) {
     using S = typename Storage<ST>::S;
     using T = typename Storage<ST>::T;
     using X = RowBox<ST>;
@@ -148,10 +148,10 @@ __global__ void __launch_bounds__(NW * 32, ST == ST_F32 ? 4 : 1)
     [[maybe_unused]] auto fetch = [&](int xb, T (&v)[LN]) {
         const S* p = rhs + g.at(0, ry, 0) + xb;
         if constexpr (sizeof(S) == 4) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+            const float4 q = *reinterpret_cast<const float4*>(p);
             v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
         } else {
-            const double2 q0 = __ldg(reinterpret_cast<const double2*>(p)), q1 = __ldg(reinterpret_cast<const double2*>(p + 2));
+            const double2 q0 = *reinterpret_cast<const double2*>(p), q1 = *reinterpret_cast<const double2*>(p + 2);
             v[0] = q0.x; v[1] = q0.y; v[2] = q1.x; v[3] = q1.y;
         }
         ry = ry + 1 == g.ny ? 0 : ry + 1;

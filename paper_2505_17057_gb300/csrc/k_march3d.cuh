@@ -39,8 +39,8 @@ constexpr int march3d_min_ctas(int pde, int levels, int st, int ty, int lean) {
 
 template <int LAT, int PDE, int LEVELS, int ST, int TY, int NSTAGE, int SRC = 0, int LEAN = LEAN_NONE, int SRM = 2, bool ONES = true>
 __global__ void __launch_bounds__((TY + 1) * 32, SRC != 0 ? 1 : march3d_min_ctas(PDE, LEVELS, ST, TY, LEAN)) k_march3d(const __grid_constant__ TmapSet maps, Geom g,
-                                                           void* __restrict__ outv, Coef<typename Storage<ST>::T> cf,
-                                                           StepExtra ex, int H, int nitems, int* __restrict__ err,
+                                                           void* outv, Coef<typename Storage<ST>::T> cf,
+                                                           StepExtra ex, int H, int nitems, int* err,
                                                            const __grid_constant__ SrcParam<typename Storage<ST>::T, SRC> sa) {
     using Tr = Storage<ST>;
     using S = typename Tr::S;

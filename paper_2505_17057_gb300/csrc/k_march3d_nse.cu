@@ -20,8 +20,8 @@ namespace {
 
 template <int ST, int TY, int NSTAGE, int MINB>
 __global__ void __launch_bounds__(TY * 32, MINB) k_march3d_nse(const __grid_constant__ TmapSet maps, Geom g,
-                                                             void* __restrict__ outv, ClassNorm<typename Storage<ST>::T> cc,
-                                                             int H, int nitems, int* __restrict__ err) {
+                                                             void* outv, ClassNorm<typename Storage<ST>::T> cc,
+                                                             int H, int nitems, int* err) {
     using Tr = Storage<ST>;
     using S = typename Tr::S;
     using T = typename Tr::T;

@@ -22,9 +22,9 @@ constexpr int kNcStride = 120;   // output columns per 2D strip
 constexpr int kNcLead = 8;       // lane 0's first column lies kNcLead columns left of the strip's output
 
 template <int ST, int LEVELS, bool SHARED, int NW, int NSTAGE>
-__global__ void __launch_bounds__(NW * 32) k_march2d_ncde(const __grid_constant__ TmapSet maps, Geom g, void* __restrict__ outv,
+__global__ void __launch_bounds__(NW * 32) k_march2d_ncde(const __grid_constant__ TmapSet maps, Geom g, void* outv,
                                                           const __grid_constant__ NcdePk<typename Storage<ST>::T, 2, LEVELS - 1, SHARED> cc,
-                                                          int H, int nitems, int* __restrict__ err) {
+                                                          int H, int nitems, int* err) {
     using S = typename Storage<ST>::S;
     using T = typename Storage<ST>::T;
     using P = Pk<T>;
@@ -230,9 +230,9 @@ cudaError_t launch2(const LaunchArgs& a) {
 
 template <int ST, int LEVELS, bool SHARED, int TY, int R, int NSTAGE, int MINB>
 __global__ void __launch_bounds__(TY / R * 32, MINB) k_march3d_ncde(const __grid_constant__ TmapSet maps, Geom g,
-                                                                  void* __restrict__ outv,
+                                                                  void* outv,
                                                                   const __grid_constant__ NcdePk<typename Storage<ST>::T, 3, LEVELS - 1, SHARED> cc,
-                                                                  int H, int nitems, int* __restrict__ err) {
+                                                                  int H, int nitems, int* err) {
     using S = typename Storage<ST>::S;
     using T = typename Storage<ST>::T;
     using P = Pk<T>;

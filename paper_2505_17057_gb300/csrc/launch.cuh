@@ -13,7 +13,11 @@
 //
 // Rule every kernel launched this way keeps: chain_wait() before its first access to global memory
 // that another kernel of the chain touches, reads and writes alike (it returns when the
-// predecessor has completed and its writes are visible, and at once if there is none).
+// predecessor has completed and its writes are visible, and at once if there is none).  Such memory is
+// read by plain loads through pointers that are not __restrict__: a read-only load (__ldg, or one the
+// compiler derives from const __restrict__) is specified only for data that nothing writes while the
+// kernel lives, and neither it nor an access to memory declared unaliased has to stay behind the
+// wait's "memory" clobber.
 #pragma once
 
 #include <cuda_runtime.h>
