@@ -41,7 +41,10 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = chained ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+    // (the error state is cleared as it is returned: left set, it would be taken for the next call's)
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Rows (planes) per work item of a marching launch: `tiles` columns of n rows are cut into equal segments

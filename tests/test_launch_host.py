@@ -1,0 +1,85 @@
+"""What the library's launchers ask of the CUDA runtime, on a runtime without a GPU
+(fake_cudart/fake_cudart.cpp, loaded in a child process before the library): errors of one call stay
+with it, and what a launch needs is set on the device that it goes to."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes as C, sys
+fake = C.CDLL({fake!r}, mode=C.RTLD_GLOBAL)
+fake.fake_launches.restype = C.c_char_p
+sys.path[:0] = [{root!r}, {tests!r}]
+import numpy as np
+import gpu_cases as G
+from paper_2505_17057_gb300 import mmfd as M
+
+def put(name, value):
+    fake.fake_set(name.encode(), value)
+
+def launches():
+    # (device, kernel, (gx, gy, gz), threads, chained, cluster) since the last call
+    out = []
+    for line in fake.fake_launches().decode().splitlines():
+        w = line.split()
+        out.append((int(w[0]), w[1], tuple(int(v) for v in w[2:5]), int(w[5]), w[7] == "1", int(w[8])))
+    fake.fake_clear()
+    return out
+
+class Solver:
+    def __init__(self, **kw):
+        self.desc = M.make_desc(**kw)
+        self.h = M.mmfd_create(self.desc)
+        self.nf = M.mmfd_get_info(self.h).nf
+        n = kw["n"]
+        self.data = [np.ones(tuple(reversed(n))) for _ in range(self.nf)]
+        self.set()
+        launches()
+    def set(self):
+        M.mmfd_set_fields(self.h, 0, [d.ctypes.data for d in self.data], M.MMFD_DEVICE, M.MMFD_DT_F64)
+    def step(self, n):
+        M.mmfd_step(self.h, n)
+        return launches()
+
+def solver(lat, pde, levels, n, storage="fp32", **more):
+    kw, _ = G.case(lat, pde, levels, n, storage)
+    kw.update(more)
+    return Solver(**kw)
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    home = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")))
+    lib = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(home, "include"), "-o", lib,
+                    os.path.join(HERE, "fake_cudart", "fake_cudart.cpp")], check=True)
+
+    def run(script):
+        env = {k: v for k, v in os.environ.items() if k != "MMFD_FORCE_KERNEL"}
+        p = subprocess.run([sys.executable, "-c", PRELUDE.format(fake=lib, root=ROOT, tests=HERE) + script],
+                           capture_output=True, text=True, timeout=300, env=env)
+        assert p.returncode == 0, p.stdout + p.stderr
+    return run
+
+
+def test_a_failed_launch_leaves_no_error_behind(fake):
+    fake("""
+for lat, pde, n in [("D2Q9", "NSE", [256, 64]), ("D2Q9", "LCDE", [200, 40]), ("D3Q19", "NCDE", [128, 9, 8]), ("D2Q9", "NCDE", [20, 2000])]:
+    s = solver(lat, pde, 2, n)
+    put("fail_next", 701)                      # out of resources
+    try:
+        s.step(1)
+        raise SystemExit("the failed launch went unnoticed")
+    except M.MMFDError as e:
+        assert e.code == M.MMFD_ERR_CUDA, e.code
+    s.set()                                    # the next calls run as if nothing had happened
+    launches()
+    assert len(s.step(1)) == 1
+""")
