@@ -148,21 +148,27 @@ cudaError_t launch(const ClusterArgs& a) {
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    static int fits = -1;   // whether the device schedules such a cluster
-    if (fits < 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem);
+    // Whether the device schedules such a cluster: asked, and the attributes set, once on every device.
+    static std::atomic<int> known[kMaxDevices];   // 0 not asked, 1 yes, 2 no
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    int fits = e == cudaSuccess && dev < kMaxDevices ? known[dev].load(std::memory_order_acquire) : 0;
+    if (e == cudaSuccess && fits == 0) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         int clusters = 0;
         cudaLaunchConfig_t top = cfg;
         top.dynamicSmemBytes = kClusterSmem;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &top);
-        if (e != cudaSuccess) cudaGetLastError();
-        fits = e == cudaSuccess && clusters > 0 ? 1 : 0;
+        fits = e == cudaSuccess && clusters > 0 ? 1 : 2;
+        if (dev < kMaxDevices) known[dev].store(fits, std::memory_order_release);
     }
-    if (!fits) return cudaErrorNotSupported;
+    if (e == cudaSuccess && fits == 2) return cudaErrorNotSupported;
     ClusterLevels gl;
     for (int i = 0; i < 3; ++i) gl.lev[i] = a.lev[i];
-    return cudaLaunchKernelEx(&cfg, kern, a.g, gl, a.cur, *static_cast<const Coef<T>*>(a.coef), a.ex, a.nsteps);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kern, a.g, gl, a.cur, *static_cast<const Coef<T>*>(a.coef), a.ex, a.nsteps);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 template <int LAT, int PDE, int LEVELS, int ST>

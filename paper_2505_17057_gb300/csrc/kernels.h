@@ -39,7 +39,8 @@ using LaunchFn = cudaError_t (*)(const LaunchArgs&);
 // A launch advancing nsteps steps of a small 2D solve in one thread-block cluster: the level buffers
 // lev[0 .. levels), level t in lev[cur]; afterwards level t + nsteps dt is in the buffer that as many
 // single steps would leave it in, level t - dt (three levels) in that one's predecessor, and the
-// other buffer is as it was.  cudaErrorNotSupported if the device does not schedule the cluster.
+// other buffer is as it was.  An error (cudaErrorNotSupported if the device does not schedule the cluster)
+// means that nothing was launched.
 struct ClusterArgs {
     Geom g;
     void* lev[3];

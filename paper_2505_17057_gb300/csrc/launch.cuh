@@ -22,11 +22,16 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <utility>
 
 namespace mmfd {
 
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Devices whose answers a launcher keeps (kernel attributes and occupancies belong to the device current
+// at the call); on one beyond them it asks every time.
+constexpr int kMaxDevices = 64;
 
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool chained,

@@ -300,11 +300,12 @@ int solver_step(Solver* s, long long nsteps) {
         c.nsteps = (int)(nsteps - done < 100000 ? nsteps - done : 100000);
         c.stream = s->stream;
         cudaError_t e = s->fn_cluster(c);
-        if (e == cudaErrorNotSupported) {
+        if (e != cudaSuccess) {
+            // nothing was launched: one launch per step from here on (an error that is not the cluster's
+            // own comes back from those)
             s->fn_cluster = nullptr;
             break;
         }
-        if (e != cudaSuccess) return cuda_fail(e, "cluster step kernel");
         s->cur = (int)((s->cur + c.nsteps) % s->nlev);
         s->steps_done += c.nsteps;
         done += c.nsteps;

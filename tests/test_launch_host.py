@@ -83,3 +83,34 @@ for lat, pde, n in [("D2Q9", "NSE", [256, 64]), ("D2Q9", "LCDE", [200, 40]), ("D
     launches()
     assert len(s.step(1)) == 1
 """)
+
+
+def test_cluster_launch_on_every_device_and_the_way_back(fake):
+    fake("""
+for dev in (0, 1, 0, 3):
+    fake.fake_device(dev)
+    for storage, pde in [("fp32", "LCDE"), ("bf16", "NSE"), ("fp64", "LCDE")]:
+        s = solver("D2Q9", pde, 2, [64, 48], storage)
+        for got in (s.step(5), s.step(2)):         # one launch for all steps of a call
+            assert len(got) == 1 and "k_cluster" in got[0][1] and got[0][0] == dev and got[0][5] == 16, got
+# a cluster that the device does not take after all: the steps run one by one, and go on doing so
+s = solver("D2Q9", "LCDE", 2, [64, 48])
+for code in (912, 701, 1):
+    put("fail_next", code)
+    got = s.step(5)
+    assert len(got) == 5 and all("k_direct" in g[1] for g in got), (code, got)
+    s = solver("D2Q9", "LCDE", 2, [64, 48])
+""")
+
+
+def test_device_without_such_clusters(fake):
+    fake("""
+put("clusters", 0)
+s = solver("D2Q9", "LCDE", 2, [64, 48])
+assert ["k_direct" in g[1] for g in s.step(3)] == [True] * 3
+fake.fake_device(1)
+put("clusters", 1)                                  # another device of the machine has room for them
+s = solver("D2Q9", "LCDE", 2, [64, 48])
+got = s.step(3)
+assert len(got) == 1 and "k_cluster" in got[0][1], got
+""")
