@@ -858,20 +858,14 @@ cudaError_t launch_march2d_t(const LaunchArgs& a) {
     constexpr int NF = pde_nf(PDE, LAT);
     constexpr size_t smem = march2d_smem<ST, LEVELS, NF, NW, NSTAGE, LN, RPS>();
     auto kern = k_march2d<LAT, PDE, LEVELS, ST, NW, NSTAGE, LN, RPS, SRC, LEAN, SRM>;
-    static int resident = 0;
-    if (resident == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
-        if (e != cudaSuccess) return e;
-        // The plain FP32 linear step is bound by DRAM, and fewer concurrent row streams are easier on it:
-        // at 8192^2 (7 CTAs fit an SM) 116 us at 7, 113 at 5, 98 at 4, 90 at 3, 117 at 2.
-        if (PDE == PDE_LCDE && ST == ST_F32 && LEVELS == 2 && SRC == 0 && per_sm > 3) per_sm = 3;
-        resident = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    static std::atomic<unsigned long long> known[kMaxDevices];
+    Fit fit;
+    const cudaError_t e = fit_of(kern, NW * 32, smem, known, &fit);
+    if (e != cudaSuccess) return e;
+    // The plain FP32 linear step is bound by DRAM, and fewer concurrent row streams are easier on it:
+    // at 8192^2 (7 CTAs fit an SM) 116 us at 7, 113 at 5, 98 at 4, 90 at 3, 117 at 2.
+    if (PDE == PDE_LCDE && ST == ST_F32 && LEVELS == 2 && SRC == 0 && fit.per_sm > 3) fit.per_sm = 3;
+    const int resident = fit.ctas();
     constexpr int COLS = 32 * LN;
     const int strips = (a.g.nx + COLS - 1) / COLS;
     int H = a.H;

@@ -200,17 +200,11 @@ cudaError_t launch_nse(const LaunchArgs& a) {
     constexpr int NSTAGE = 3;
     constexpr size_t smem = tbn_smem<ST, NW, NSTAGE>();
     auto kern = k_march2d_nse<ST, TT, NW, NSTAGE>;
-    static int resident = 0;
-    if (resident == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
-        if (e != cudaSuccess) return e;
-        resident = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    static std::atomic<unsigned long long> known[kMaxDevices];
+    Fit fit;
+    const cudaError_t e = fit_of(kern, NW * 32, smem, known, &fit);
+    if (e != cudaSuccess) return e;
+    const int resident = fit.ctas();
     const int strips = (a.g.nx + kTbnLead / 2 + kTbnStride - 1) / kTbnStride;
     int H = a.H;
     if (H <= 0) H = march_height(strips, a.g.ny, (long long)resident * NW, 2 * TT, TT == 1 ? 2 : 8, 512);

@@ -285,17 +285,11 @@ cudaError_t launch(const LaunchArgs& a) {
     constexpr int NW = 4;
     constexpr size_t smem = RowBox<ST>::smem(NW);
     auto kern = k_theta<LAT, ST, TT, FIRST, NW>;
-    static int resident = 0;
-    if (resident == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
-        if (e != cudaSuccess) return e;
-        resident = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    static std::atomic<unsigned long long> known[kMaxDevices];
+    Fit fit;
+    const cudaError_t e = fit_of(kern, NW * 32, smem, known, &fit);
+    if (e != cudaSuccess) return e;
+    const int resident = fit.ctas();
     constexpr int STRIDE = FIRST ? 128 : kThStride, LEAD = FIRST ? 0 : kThLead;
     const int strips = (a.g.nx + LEAD / 2 + STRIDE - 1) / STRIDE;
     int H = a.H;

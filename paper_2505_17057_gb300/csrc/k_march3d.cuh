@@ -435,23 +435,15 @@ cudaError_t launch_march3d_t(const LaunchArgs& a) {
     if constexpr (kAligned) {
         if (aligned) kern = k_march3d<LAT, PDE, LEVELS, ST, TY, NSTAGE, SRC, LEAN, SRM, false>;
     }
-    static int resident_of[2] = {0, 0}, sms = 0, l2 = 0;
-    int& fit = resident_of[aligned];
-    if (fit == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);
-        if (e != cudaSuccess) return e;
-        fit = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    static std::atomic<unsigned long long> known[2][kMaxDevices];
+    Fit fit;
+    const cudaError_t e = fit_of(kern, THREADS, smem, known[aligned], &fit);
+    if (e != cudaSuccess) return e;
     // Two FP32 levels larger than L2 stream through DRAM, which fewer concurrent plane streams suit better:
     // 512^3 174 us with two CTAs per SM against 215 with three; 256^3, in L2, 28.5 against 26.1.
-    const bool streams = kAligned && ST == ST_F32 && LEVELS == 2 && 2 * a.g.fs * (long long)sizeof(T) > l2;
-    const int resident = streams && fit > 2 * sms ? 2 * sms : fit;
+    const bool streams = kAligned && ST == ST_F32 && LEVELS == 2 && 2 * a.g.fs * (long long)sizeof(T) > fit.l2;
+    if (streams && fit.per_sm > 2) fit.per_sm = 2;
+    const int resident = fit.ctas();
     int H = 0, nitems = 0, grid = 0;
     march3d_split(a.g, TY, a.H, resident, TY == kLeanWideRows && ST == ST_BF16, &H, &nitems, &grid);
     SrcParam<T, SRC> sa{};

@@ -113,17 +113,11 @@ cudaError_t launch(const LaunchArgs& a) {
     constexpr size_t smem = ring_smem<ST, 2, 4, TY, NSTAGE>();
     constexpr int THREADS = TY * 32;
     auto kern = k_march3d_nse<ST, TY, NSTAGE, MINB>;
-    static int resident = 0;
-    if (resident == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);
-        if (e != cudaSuccess) return e;
-        resident = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    static std::atomic<unsigned long long> known[kMaxDevices];
+    Fit fit;
+    const cudaError_t e = fit_of(kern, THREADS, smem, known, &fit);
+    if (e != cudaSuccess) return e;
+    const int resident = fit.ctas();
     int H = 0, nitems = 0, grid = 0;
     march3d_split(a.g, TY, a.H, resident, false, &H, &nitems, &grid);
     return launch_chained(kern, grid, THREADS, smem, a.stream, a.chained, *a.maps, a.g, a.out,

@@ -204,17 +204,11 @@ cudaError_t launch2(const LaunchArgs& a) {
     constexpr int SLOT = ((2 * (128 + 2 * (16 / ES)) * ES + 127) / 128) * 128;
     constexpr size_t smem = 128 + 128 * ((NW * NSTAGE * 8 + 127) / 128) + (size_t)NW * NSTAGE * (LEVELS - 1) * SLOT;
     auto kern = k_march2d_ncde<ST, LEVELS, SHARED, NW, NSTAGE>;
-    static int resident = 0;
-    if (resident == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
-        if (e != cudaSuccess) return e;
-        resident = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    static std::atomic<unsigned long long> known[kMaxDevices];
+    Fit fit;
+    const cudaError_t e = fit_of(kern, NW * 32, smem, known, &fit);
+    if (e != cudaSuccess) return e;
+    const int resident = fit.ctas();
     const int strips = (a.g.nx + kNcLead / 2 + kNcStride - 1) / kNcStride;
     int H = a.H;
     if (H <= 0) H = march_height(strips, a.g.ny, (long long)resident * NW, 2, 2, 256);
@@ -386,17 +380,11 @@ cudaError_t launch3(const LaunchArgs& a) {
     constexpr size_t smem = ring_smem<ST, LEVELS, 1, TY, NSTAGE>();
     constexpr int THREADS = TY / R * 32;
     auto kern = k_march3d_ncde<ST, LEVELS, SHARED, TY, R, NSTAGE, MINB>;
-    static int resident = 0;
-    if (resident == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);
-        if (e != cudaSuccess) return e;
-        resident = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    static std::atomic<unsigned long long> known[kMaxDevices];
+    Fit fit;
+    const cudaError_t e = fit_of(kern, THREADS, smem, known, &fit);
+    if (e != cudaSuccess) return e;
+    const int resident = fit.ctas();
     int H = 0, nitems = 0, grid = 0;
     march3d_split(a.g, TY, a.H, resident, false, &H, &nitems, &grid);
     return launch_chained(kern, grid, THREADS, smem, a.stream, a.chained,

@@ -52,6 +52,40 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
     return e;
 }
 
+// CTAs of a kernel that an SM holds, the device's SMs and its L2 bytes.
+struct Fit {
+    int per_sm, sms;
+    long long l2;
+    int ctas() const { return per_sm * sms; }
+};
+
+// The Fit of `kern` at `threads` threads and `smem` bytes of dynamic shared memory a CTA on the current
+// device, its shared memory limit raised on the way.  Asked once per device and kept in `known`, one word
+// per device, so that concurrent host threads see either nothing or the whole answer.
+template <typename... P>
+cudaError_t fit_of(void (*kern)(P...), int threads, size_t smem, std::atomic<unsigned long long> (&known)[kMaxDevices], Fit* f) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    unsigned long long w = e == cudaSuccess && dev < kMaxDevices ? known[dev].load(std::memory_order_acquire) : 0;
+    if (e == cudaSuccess && w == 0) {
+        int per_sm = 0, sms = 0, l2 = 0;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+        if (e == cudaSuccess) {
+            w = (unsigned long long)l2 << 32 | (unsigned long long)sms << 8 | (unsigned long long)(per_sm > 0 ? per_sm : 1);
+            if (dev < kMaxDevices) known[dev].store(w, std::memory_order_release);
+        }
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+    }
+    *f = {(int)(w & 255), (int)(w >> 8 & 0xffffff), (long long)(w >> 32)};
+    return cudaSuccess;
+}
+
 // Rows (planes) per work item of a marching launch: `tiles` columns of n rows are cut into equal segments
 // of at least hmin and at most hmax rows, dealt round-robin to `slots` warps (CTAs), each segment
 // streamed with `halo` further rows.  Picks the cut whose longest queue streams the fewest rows: for

@@ -114,3 +114,29 @@ s = solver("D2Q9", "LCDE", 2, [64, 48])
 got = s.step(3)
 assert len(got) == 1 and "k_cluster" in got[0][1], got
 """)
+
+
+@pytest.mark.parametrize("lat,pde,levels,n,more", [
+    ("D3Q19", "NSE", 2, [96, 20, 18], dict(dx=[1.0] * 3, a=(1.0, 0.0, 0.0), abar=(1.0, 0.0, 0.0))),
+    ("D3Q19", "NCDE", 3, [70, 20, 18], dict(dx=[1.0] * 3)),
+    ("D3Q19", "NSE", 2, [128, 20, 18], {}),
+    ("D3Q7", "LCDE", 2, [256, 64, 20], {}),
+    ("D2Q9", "NSE", 2, [256, 64], dict(dx=[1.0] * 2, a=(1.0, 0.0, 0.0), abar=(1.0, 0.0, 0.0), temporal_depth=3)),
+    ("D2Q9", "NCDE", 2, [256, 64], dict(temporal_depth=1)),
+    ("D2Q9", "LCDE", 2, [256, 64], dict(storage="fp64", temporal_depth=2)),
+])
+def test_marching_kernels_on_every_device(fake, lat, pde, levels, n, more):
+    fake(f"""
+kw = dict(flags=M.MMFD_FLAG_ALLOW_UNSTABLE, **{more!r})
+storage = kw.pop("storage", "fp32")
+grids = set()
+for dev in (0, 1, 2, 0):
+    fake.fake_device(dev)
+    got = solver({lat!r}, {pde!r}, {levels}, {n!r}, storage, **kw).step(3)
+    assert got and all(g[0] == dev and "k_march" in g[1] for g in got), got
+    grids.add(tuple(g[1:] for g in got))
+assert len(grids) == 1, grids
+# as does a device that the library keeps no answer for
+fake.fake_device(100)
+assert solver({lat!r}, {pde!r}, {levels}, {n!r}, storage, **kw).step(3)
+""")
