@@ -239,7 +239,9 @@ int mmfd_desc_init(mmfd_desc* d);
  * the environment variable MMFD_FORCE_KERNEL=direct before mmfd_create selects the direct
  * kernel for any grid, MMFD_FORCE_KERNEL=generic the general pair form,
  * MMFD_FORCE_KERNEL=lean3d_rows16 / lean3d_rows4 the 3D lean tile (for comparisons; all compute
- * the same update). */
+ * the same update).  MMFD_FORCE_KERNEL=cluster refuses a solver that does not step with the cluster
+ * kernel (small 2D grids, two or more steps per call; it reports k_direct's name, whose bits it
+ * computes), and such a solver's step fails where it would go back to one launch per step. */
 int mmfd_create(const mmfd_desc* desc, mmfd_solver** out);
 
 /* Copy one level into the solver.  level 0 = t_n, level 1 = t_{n-1} (three-level only).

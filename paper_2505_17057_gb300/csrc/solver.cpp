@@ -114,7 +114,13 @@ int solver_init_device(Solver* s) {
     cudaError_t e = cudaMemsetAsync(s->d_flag, 0, 256, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     s->cur = 0;
-    return solver_pick_kernels(s);
+    rc = solver_pick_kernels(s);
+    if (rc != MMFD_OK) return rc;
+    // (the cluster kernel reports the direct kernel's name, whose bits it computes)
+    const char* force = std::getenv("MMFD_FORCE_KERNEL");
+    s->need_cluster = force && std::strcmp(force, "cluster") == 0;
+    if (s->need_cluster && !s->fn_cluster) return set_error(MMFD_ERR_UNSUPPORTED, "this solver does not step with the cluster kernel");
+    return MMFD_OK;
 }
 
 void solver_free_device(Solver* s) {
@@ -300,6 +306,7 @@ int solver_step(Solver* s, long long nsteps) {
         c.nsteps = (int)(nsteps - done < 100000 ? nsteps - done : 100000);
         c.stream = s->stream;
         cudaError_t e = s->fn_cluster(c);
+        if (e != cudaSuccess && s->need_cluster) return cuda_fail(e, "cluster step kernel");
         if (e != cudaSuccess) {
             // nothing was launched: one launch per step from here on (an error that is not the cluster's
             // own comes back from those)

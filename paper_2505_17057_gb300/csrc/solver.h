@@ -31,6 +31,7 @@ struct Solver {
     int max_depth = 1;                           // deepest blocking this solver's ghosts allow
     LaunchFn fn = nullptr;                       // single-step kernel
     ClusterFn fn_cluster = nullptr;              // all steps of a call in one launch (small grids)
+    bool need_cluster = false;                   // MMFD_FORCE_KERNEL=cluster: an error instead of the way back
     LaunchFn fn_block = nullptr;                 // temporally blocked kernel (depth > 1)
     int variant = 0;
     const char* kernel_name = "k_direct";

@@ -140,3 +140,40 @@ assert len(grids) == 1, grids
 fake.fake_device(100)
 assert solver({lat!r}, {pde!r}, {levels}, {n!r}, storage, **kw).step(3)
 """)
+
+
+def test_cluster_on_request_only_where_the_rule_takes_it(fake):
+    fake("""
+import os
+os.environ["MMFD_FORCE_KERNEL"] = "cluster"
+
+def takes(lat, pde, levels, n, storage, **more):
+    try:
+        s = solver(lat, pde, levels, n, storage, **more)
+    except M.MMFDError as e:
+        assert e.code == M.MMFD_ERR_UNSUPPORTED, e
+        return False
+    assert "k_cluster" in s.step(2)[0][1]
+    put("fail_next", 912)
+    try:
+        s.step(2)
+    except M.MMFDError as e:
+        assert e.code == M.MMFD_ERR_CUDA
+        return True
+    raise SystemExit("went back to one launch per step in silence")
+
+for lat, pde, levels in [c for c in G.SUPPORTED if c[0].startswith("D2")]:
+    cost = {"LCDE": 2, "NCDE": 3, "NSE": 5}[pde] * (levels - 1)
+    for storage in ("fp64", "fp32", "bf16"):
+        f64 = storage == "fp64"
+        if f64 and pde != "LCDE":
+            assert not takes(lat, pde, levels, [16, 16], storage)
+            continue
+        most = 65536 // (cost * (5 if f64 else 1))
+        assert takes(lat, pde, levels, [100, 33] if most >= 3300 else [100, most // 100], storage), (lat, pde, levels, storage)
+        assert takes(lat, pde, levels, [127, most // 127], storage), (lat, pde, levels, storage)
+        assert not takes(lat, pde, levels, [127, most // 127 + 1], storage), (lat, pde, levels, storage)
+assert not takes("D2Q9", "LCDE", 2, [128, 16], "fp32")          # the marching kernels' widths
+assert not takes("D3Q7", "LCDE", 2, [16, 16, 4], "fp32")
+assert not takes("D2Q9", "LCDE", 2, [32, 16], "fp32", boundary="dirichlet")
+""")
