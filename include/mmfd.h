@@ -376,9 +376,10 @@ int mmfd_wave_coefficients(double gamma, double a[3], double ahat[3]);
  * 4, 8, 16, 32, 64, 128 (2D) or 0, 8, 16, 32, 64, 128 (3D marching kernels) -- and keeps the fastest for
  * later mmfd_step calls.  Trial launches read the current level(s) and write only the spare
  * buffer, so the solver's fields and step count are unchanged; the call synchronises the
- * solver's stream.  Any solver can be tuned, before or after its fields are set.
+ * solver's stream.  Trials are launched as steps are; a small 2D solve, all of whose steps run in one
+ * launch, has nothing to choose and is only timed.  Any solver can be tuned, before or after its fields are set.
  * cache_path (NULL = no cache): a text file of earlier choices, one line per key
- * (device name, SM count, lattice, PDE, levels, storage, flags, grid, depth mode).  A hit applies
+ * (device name, SM count, lattice, PDE, levels, storage, flags, grid, depth mode, launch mode).  A hit applies
  * the stored choice without timing; a miss times the candidates and appends the choice.  A
  * cache that cannot be read or written is ignored (the tuning result still applies). */
 typedef struct {

@@ -26,6 +26,7 @@ constexpr size_t kClusterSmem = 227 * 1024;
 
 struct ClusterLevels {
     void* lev[3];
+    void* out[3];
 };
 
 // Rows per CTA, and bytes of shared memory of a CTA holding nlev levels.
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_cluster(Geom g, const __gri
     for (int l = 0; l < NLEV - 1; ++l) {
         const int b = l == 0 ? c : (c + 2) % 3;
         for (int f = 0; f < NF; ++f) {
-            S* p = static_cast<S*>(gl.lev[b]) + f * g.fs;
+            S* p = static_cast<S*>(gl.out[b]) + f * g.fs;
             const S* q = sm + b * lvl + f * gs.fs;
             for (int i = threadIdx.x; i < rows * (int)g.py; i += kClusterThreads) {
                 const int y = i / (int)g.py, x = i - y * (int)g.py;   // padded column
@@ -165,7 +166,10 @@ cudaError_t launch(const ClusterArgs& a) {
     }
     if (e == cudaSuccess && fits == 2) return cudaErrorNotSupported;
     ClusterLevels gl;
-    for (int i = 0; i < 3; ++i) gl.lev[i] = a.lev[i];
+    for (int i = 0; i < 3; ++i) {
+        gl.lev[i] = a.lev[i];
+        gl.out[i] = a.out[i];
+    }
     if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kern, a.g, gl, a.cur, *static_cast<const Coef<T>*>(a.coef), a.ex, a.nsteps);
     if (e != cudaSuccess) cudaGetLastError();
     return e;

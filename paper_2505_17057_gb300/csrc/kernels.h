@@ -44,6 +44,7 @@ using LaunchFn = cudaError_t (*)(const LaunchArgs&);
 struct ClusterArgs {
     Geom g;
     void* lev[3];
+    void* out[3];          // where the levels are written back, by the same indices: lev, or a spare buffer to time a launch
     int cur;
     const void* coef;
     StepExtra ex;          // step: that of the first new level

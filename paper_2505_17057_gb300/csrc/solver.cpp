@@ -241,12 +241,27 @@ void solver_launch_args(Solver* s, LaunchArgs& a) {
     }
 }
 
-int solver_step(Solver* s, long long nsteps) {
-    if (!s->fields_set) return set_error(MMFD_ERR_STATE, "set the fields before stepping");
-    // steps of a captured stream keep the plain dependencies of the capture
+void solver_cluster_args(Solver* s, int nsteps, ClusterArgs& c) {
+    c.g = s->g;
+    for (int i = 0; i < 3; ++i) c.lev[i] = c.out[i] = s->lev[i];
+    c.cur = s->cur;
+    c.coef = s->coef();
+    c.ex.seed = s->desc.seed;
+    c.ex.step = s->steps_done + 1;
+    c.ex.sr = (s->r.st == ST_BF16 && (s->desc.flags & MMFD_FLAG_STOCHASTIC_ROUND)) ? 1 : 0;
+    c.nsteps = nsteps;
+    c.stream = s->stream;
+}
+
+void solver_chain(Solver* s) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
     if (cudaStreamIsCapturing(s->stream, &cap) != cudaSuccess) cudaGetLastError();
     s->chained = cap == cudaStreamCaptureStatusNone;
+}
+
+int solver_step(Solver* s, long long nsteps) {
+    if (!s->fields_set) return set_error(MMFD_ERR_STATE, "set the fields before stepping");
+    solver_chain(s);
     if (s->r.theta_on) {
         // Eq. (GCN): rhs = ((1 - theta) I + theta E) phi^n, then r.sweeps Jacobi sweeps from
         // x = phi^n, each into the spare level buffer
@@ -296,15 +311,7 @@ int solver_step(Solver* s, long long nsteps) {
     long long done = 0;
     while (s->fn_cluster && nsteps - done >= 2) {
         ClusterArgs c;
-        c.g = s->g;
-        for (int i = 0; i < 3; ++i) c.lev[i] = s->lev[i];
-        c.cur = s->cur;
-        c.coef = s->coef();
-        c.ex.seed = s->desc.seed;
-        c.ex.step = s->steps_done + 1;
-        c.ex.sr = (s->r.st == ST_BF16 && (s->desc.flags & MMFD_FLAG_STOCHASTIC_ROUND)) ? 1 : 0;
-        c.nsteps = (int)(nsteps - done < 100000 ? nsteps - done : 100000);
-        c.stream = s->stream;
+        solver_cluster_args(s, (int)(nsteps - done < 100000 ? nsteps - done : 100000), c);
         cudaError_t e = s->fn_cluster(c);
         if (e != cudaSuccess && s->need_cluster) return cuda_fail(e, "cluster step kernel");
         if (e != cudaSuccess) {

@@ -38,7 +38,7 @@ struct Solver {
     int tile_rows = 0;  // 3D marching kernels: rows of the CTA tile (mmfd_info_t::tile_rows)
     int* d_flag = nullptr;                       // device error flag written by kernels
     bool fields_set = false;
-    bool chained = false;                        // this mmfd_step call launches its steps chained (launch.cuh)
+    bool chained = false;                        // this call launches its steps chained (launch.cuh)
     bool use_tma = false;                        // kernel family consumes tensor maps
     int lean = 0;                                // LEAN_* variant of the marching kernel in use
     CUtensorMap tmaps[3][4];                     // per level buffer, per field
@@ -81,6 +81,11 @@ int solver_pick_kernels(Solver* s);
 int solver_check_flag(Solver* s);
 // Launch arguments of the next step: inputs the current level(s), output the spare buffer.
 void solver_launch_args(Solver* s, LaunchArgs& a);
+// The same for the cluster kernel.
+void solver_cluster_args(Solver* s, int nsteps, ClusterArgs& c);
+// Whether this call's steps are launched chained: yes, except that steps of a captured stream keep the plain
+// dependencies of the capture.
+void solver_chain(Solver* s);
 // Switch to temporal depth `depth` (1 = unblocked; must not exceed max_depth).
 void solver_use_depth(Solver* s, int depth);
 // Time the candidate configurations and keep the fastest (mmfd_autotune).

@@ -27,7 +27,8 @@ std::string tune_key(const Solver* s) {
     std::ostringstream k;
     k << name << ":" << sms << ":lat" << s->r.lat << ":pde" << s->r.pde << ":lev" << s->r.levels << ":st" << s->r.st
       << ":fl" << s->desc.flags << ":n" << s->g.nx << "x" << s->g.ny << "x" << s->g.nz << ":depth"
-      << (s->desc.temporal_depth == 0 ? std::string("auto") : std::to_string(s->depth));
+      << (s->desc.temporal_depth == 0 ? std::string("auto") : std::to_string(s->depth))
+      << ":chained";   // timings of unchained launches, under the key without it, do not carry over
     return k.str();
 }
 
@@ -77,6 +78,7 @@ int solver_autotune(Solver* s, const char* cache_path, mmfd_tune_info* out) {
         return MMFD_OK;
     }
 
+    solver_chain(s);   // trials are launched as steps are
     std::vector<int> depths;
     if (auto_depth)
         for (int d = 1; d <= s->max_depth; ++d) depths.push_back(d);
@@ -111,6 +113,33 @@ int solver_autotune(Solver* s, const char* cache_path, mmfd_tune_info* out) {
         if (e2 == cudaSuccess) e2 = cudaEventElapsedTime(ms, e0, e1);
         return e2;
     };
+    // a small grid's steps run in cluster launches, which have nothing to choose: only their time is taken,
+    // of launches that write the levels back into the spare buffer
+    if (s->fn_cluster) {
+        const int n = 64;
+        ClusterArgs c;
+        solver_cluster_args(s, n, c);
+        for (int i = 0; i < 3; ++i) c.out[i] = s->lev[s->next()];
+        float t[4] = {0.f, 0.f, 0.f, 0.f};   // (the first one warms up)
+        for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
+            e = cudaEventRecord(e0, s->stream);
+            if (e == cudaSuccess) e = s->fn_cluster(c);
+            if (e == cudaSuccess) e = cudaEventRecord(e1, s->stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&t[k], e0, e1);
+        }
+        if (e == cudaSuccess) {
+            best = (double)std::max(std::min(t[1], t[2]), std::min(std::max(t[1], t[2]), t[3])) / n;
+            best_d = 1;
+            best_h = 0;
+            info.candidates = 1;
+            depths.clear();
+        } else {
+            if (s->need_cluster) rc = cuda_fail(e, "autotune trial launch");
+            s->fn_cluster = nullptr;   // as a step would: one launch per step
+            if (rc != MMFD_OK) depths.clear();
+        }
+    }
     for (int d : depths) {
         solver_use_depth(s, d);
         LaunchFn fn = d >= 2 ? s->fn_block : s->fn;

@@ -45,3 +45,26 @@ def test_cluster_runs_and_equals_the_direct_kernel(mm, monkeypatch, lat, pde, le
         a = run(mm, monkeypatch, "cluster", kw, fields, [4, 3])
         b = run(mm, monkeypatch, "direct", kw, fields, [7])
         assert all(np.array_equal(p, q) for x, y in zip(a, b) for p, q in zip(x, y)), n
+
+
+@pytest.mark.parametrize("lat,pde,levels,storage", [("D2Q9", "NSE", 2, "fp32"), ("D2Q9", "LCDE", 3, "fp64"),
+                                                    ("D2Q9", "NCDE", 3, "bf16")])
+def test_autotuning_a_cluster_solver_leaves_its_levels(mm, monkeypatch, tmp_path, lat, pde, levels, storage):
+    monkeypatch.setenv("MMFD_FORCE_KERNEL", "cluster")
+    kw, prob = G.case(lat, pde, levels, [90, 25], storage)
+    fields = G.random_level(prob, np.random.default_rng(3))
+    s, plain = mm.Solver(mm.make_desc(**kw)), mm.Solver(mm.make_desc(**kw))
+    try:
+        for x in (s, plain):
+            x.set_fields(fields)
+            x.step(3)
+        info = s.autotune(str(tmp_path / "tune.txt"))
+        assert info.candidates == 1 and info.ms_per_step > 0 and s.get_info().steps_done == 3
+        for steps in (0, 4):
+            s.step(steps)
+            plain.step(steps)
+            for l in range(levels - 1):
+                assert all(np.array_equal(a, b) for a, b in zip(s.fields(l), plain.fields(l))), (steps, l)
+    finally:
+        s.close()
+        plain.close()

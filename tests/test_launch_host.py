@@ -177,3 +177,23 @@ assert not takes("D2Q9", "LCDE", 2, [128, 16], "fp32")          # the marching k
 assert not takes("D3Q7", "LCDE", 2, [16, 16, 4], "fp32")
 assert not takes("D2Q9", "LCDE", 2, [32, 16], "fp32", boundary="dirichlet")
 """)
+
+
+def test_autotuner_times_the_launches_that_steps_make(fake):
+    fake("""
+for lat, pde, levels, n, kernel in [("D2Q9", "NCDE", 2, [200, 40], "k_march2d"), ("D3Q19", "NSE", 2, [40, 9, 8], "k_direct"),
+                                    ("D2Q9", "LCDE", 2, [64, 48], "k_cluster"), ("D2Q5", "LCDE", 3, [64, 48], "k_cluster")]:
+    s = solver(lat, pde, levels, n)
+    for before in (0, 2):                          # tuned before the first step, and after one
+        if before:
+            assert all(kernel in g[1] for g in s.step(before))
+        info = M.mmfd_autotune(s.h)
+        got = launches()
+        assert info.candidates >= 1 and got
+        # trials are programmatic dependents, as steps are (the cluster's one launch depends on nothing)
+        assert all(kernel in g[1] and g[4] == (kernel != "k_cluster") for g in got), got[:3]
+        if kernel == "k_cluster":
+            assert (info.temporal_depth, info.rows_per_item, info.candidates) == (1, 0, 1)
+            assert abs(info.ms_per_step - 1.0 / 64) < 1e-9     # the fake events lie 1 ms apart
+    assert all(kernel in g[1] for g in s.step(2))
+""")
