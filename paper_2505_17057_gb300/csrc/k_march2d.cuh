@@ -862,9 +862,15 @@ cudaError_t launch_march2d_t(const LaunchArgs& a) {
     Fit fit;
     const cudaError_t e = fit_of(kern, NW * 32, smem, known, &fit);
     if (e != cudaSuccess) return e;
-    // The plain FP32 linear step is bound by DRAM, and fewer concurrent row streams are easier on it:
-    // at 8192^2 (7 CTAs fit an SM) 116 us at 7, 113 at 5, 98 at 4, 90 at 3, 117 at 2.
-    if (PDE == PDE_LCDE && ST == ST_F32 && LEVELS == 2 && SRC == 0 && fit.per_sm > 3) fit.per_sm = 3;
+    // The plain two-level FP32 linear step takes seven CTAs per SM, but is bound by memory, and fewer
+    // concurrent row streams are easier on it: four, or three once its two levels are well beyond L2.  us per
+    // step at seven / four / three: 768^2 2.98 / 2.99 / 3.19, 1024^2 3.93 / 3.63 / 3.75, 2048^2 8.26 / 7.64 /
+    // 7.42, 3584^2 19.6 / 19.0 / 18.9, 4096^2 (1.0 of L2) 26.7 / 23.8 / 24.6, 4608^2 (1.26 of it) 28.8 / 28.1 /
+    // 30.9, 5120^2 (1.55) 38.7 / 37.7 / 36.7, 6144^2 58.0 / 57.0 / 51.3, 8192^2 101.7 / 98.2 / 89.8 (two: 117).
+    if (PDE == PDE_LCDE && ST == ST_F32 && LEVELS == 2 && SRC == 0) {
+        const int most = 4 * a.g.fs * (long long)sizeof(T) > 3 * fit.l2 ? 3 : 4;
+        if (fit.per_sm > most) fit.per_sm = most;
+    }
     const int resident = fit.ctas();
     constexpr int COLS = 32 * LN;
     const int strips = (a.g.nx + COLS - 1) / COLS;

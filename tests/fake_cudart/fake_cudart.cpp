@@ -22,7 +22,7 @@ thread_local cudaError_t last = cudaSuccess;
 thread_local dim3 cfg_grid, cfg_block;
 thread_local size_t cfg_smem;
 thread_local void* cfg_stream;
-int ctas_per_sm = 7, clusters = 1, capturing = 0, fail_next = 0, occupancy_calls = 0;
+int ctas_per_sm = 7, clusters = 1, capturing = 0, fail_next = 0, sms = 152, l2_kb = 129 << 10;
 float event_ms = 1.0f;
 
 cudaError_t fail(cudaError_t e) {
@@ -58,8 +58,9 @@ void fake_set(const char* what, int v) {
     else if (!std::strcmp(what, "clusters")) clusters = v;
     else if (!std::strcmp(what, "capturing")) capturing = v;
     else if (!std::strcmp(what, "fail_next")) fail_next = v;
+    else if (!std::strcmp(what, "sms")) sms = v;
+    else if (!std::strcmp(what, "l2_kb")) l2_kb = v;
 }
-int fake_occupancy_calls() { return occupancy_calls; }
 void fake_clear() { launches.clear(); }
 const char* fake_launches() { return launches.c_str(); }
 
@@ -99,8 +100,6 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute at, int v) {
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {
-    std::lock_guard<std::recursive_mutex> l(mu);
-    ++occupancy_calls;
     *n = ctas_per_sm;
     return cudaSuccess;
 }
@@ -109,7 +108,7 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
 // ---- device
 cudaError_t cudaGetDevice(int* d) { *d = device; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
-    *v = a == cudaDevAttrMultiProcessorCount ? 152 : a == cudaDevAttrL2CacheSize ? 129 << 20 : 0;
+    *v = a == cudaDevAttrMultiProcessorCount ? sms : a == cudaDevAttrL2CacheSize ? l2_kb << 10 : 0;
     return cudaSuccess;
 }
 cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) { std::memset(p, 0, sizeof(*p)); std::strcpy(p->name, "fake"); return cudaSuccess; }

@@ -197,3 +197,28 @@ for lat, pde, levels, n, kernel in [("D2Q9", "NCDE", 2, [200, 40], "k_march2d"),
             assert abs(info.ms_per_step - 1.0 / 64) < 1e-9     # the fake events lie 1 ms apart
     assert all(kernel in g[1] for g in s.step(2))
 """)
+
+
+def test_ctas_per_sm_of_the_plain_linear_step(fake):
+    # (4 SMs and 1 MB of L2, so that small grids fill the GPU)
+    fake("""
+put("sms", 4)
+put("l2_kb", 1024)
+
+def ctas(lat, levels, n, storage="fp32"):
+    grid = solver(lat, "LCDE", levels, n, storage, temporal_depth=1).step(1)[0][2]
+    assert grid[1] == grid[2] == 1
+    return -(-grid[0] // 4)                            # (equal segments may leave part of the last round idle)
+
+for lat in ("D2Q5", "D2Q9"):
+    # at 7 CTAs per SM that fit: four while two levels stay below 1.5 times the L2, three beyond
+    assert ctas(lat, 2, [200, 256]) == 4               # 0.4 MB
+    assert ctas(lat, 2, [256, 700]) == 4               # 1.44 MB
+    assert ctas(lat, 2, [256, 800]) == 3               # 1.64 MB
+    assert ctas(lat, 2, [700, 800]) == 3
+    for levels, storage in [(2, "fp64"), (2, "bf16"), (3, "fp32")]:
+        assert ctas(lat, levels, [256, 700], storage) == 7
+put("ctas_per_sm", 2)                                  # a device with room for fewer (another one: kept per device)
+fake.fake_device(1)
+assert ctas("D2Q9", 2, [256, 800]) == 2
+""")
