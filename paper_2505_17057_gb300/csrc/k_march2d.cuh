@@ -862,20 +862,28 @@ cudaError_t launch_march2d_t(const LaunchArgs& a) {
     Fit fit;
     const cudaError_t e = fit_of(kern, NW * 32, smem, known, &fit);
     if (e != cudaSuccess) return e;
-    // The plain two-level FP32 linear step takes seven CTAs per SM, but is bound by memory, and fewer
-    // concurrent row streams are easier on it: four, or three once its two levels are well beyond L2.  us per
-    // step at seven / four / three: 768^2 2.98 / 2.99 / 3.19, 1024^2 3.93 / 3.63 / 3.75, 2048^2 8.26 / 7.64 /
-    // 7.42, 3584^2 19.6 / 19.0 / 18.9, 4096^2 (1.0 of L2) 26.7 / 23.8 / 24.6, 4608^2 (1.26 of it) 28.8 / 28.1 /
-    // 30.9, 5120^2 (1.55) 38.7 / 37.7 / 36.7, 6144^2 58.0 / 57.0 / 51.3, 8192^2 101.7 / 98.2 / 89.8 (two: 117).
-    if (PDE == PDE_LCDE && ST == ST_F32 && LEVELS == 2 && SRC == 0) {
-        const int most = 4 * a.g.fs * (long long)sizeof(T) > 3 * fit.l2 ? 3 : 4;
-        if (fit.per_sm > most) fit.per_sm = most;
-    }
-    const int resident = fit.ctas();
     constexpr int COLS = 32 * LN;
     const int strips = (a.g.nx + COLS - 1) / COLS;
+    auto height = [&](int per_sm) { return march_height(strips, a.g.ny, (long long)per_sm * fit.sms * NW, 2, 2, 256); };
+    // The plain two-level FP32 linear step takes seven CTAs per SM, but is bound by memory, and fewer
+    // concurrent row streams are easier on it: three once its two levels are well beyond L2, below that four,
+    // or three where the longest queue of stages is no longer for it (a stage is two rows, so an item of three
+    // rows takes as long as one of four).  us per step at seven / four / three: 768^2 2.98 / 2.99 / 3.19, 900^2
+    // 3.72 / 3.55 / 3.31, 1024^2 3.93 / 3.63 / 3.75, 1100^2 4.43 / 4.21 / 3.86, 1700^2 7.1 / 5.8 / 6.2, 2048^2
+    // 8.26 / 7.64 / 7.42, 3000^2 14.3 / 13.1 / 13.9, 4096^2 (1.0 of L2) 26.7 / 23.8 / 24.6, 4608^2 (1.26 of
+    // it) 28.8 / 28.1 / 30.9, 5120^2 (1.55) 38.7 / 37.7 / 36.7, 8192^2 101.7 / 98.2 / 89.8 (two: 117).
+    if (PDE == PDE_LCDE && ST == ST_F32 && LEVELS == 2 && SRC == 0 && fit.per_sm > 3) {
+        auto queue = [&](int per_sm) {   // stages of the longest queue
+            const int h = height(per_sm);
+            const long long items = (long long)strips * ((a.g.ny + h - 1) / h), slots = (long long)per_sm * fit.sms * NW;
+            return (items + slots - 1) / slots * ((h + 3) / 2);
+        };
+        const bool beyond = 4 * a.g.fs * (long long)sizeof(T) > 3 * fit.l2;
+        fit.per_sm = beyond || (a.H <= 0 && queue(3) <= queue(4)) ? 3 : 4;
+    }
+    const int resident = fit.ctas();
     int H = a.H;
-    if (H <= 0) H = march_height(strips, a.g.ny, (long long)resident * NW, 2, 2, 256);
+    if (H <= 0) H = height(fit.per_sm);
     const int nitems = strips * ((a.g.ny + H - 1) / H);
     const int blocks_needed = (nitems + NW - 1) / NW;
     const int grid = blocks_needed < resident ? blocks_needed : resident;

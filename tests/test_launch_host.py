@@ -218,6 +218,17 @@ for lat in ("D2Q5", "D2Q9"):
     assert ctas(lat, 2, [700, 800]) == 3
     for levels, storage in [(2, "fp64"), (2, "bf16"), (3, "fp32")]:
         assert ctas(lat, levels, [256, 700], storage) == 7
+# below that also three where they queue no more stages than four.  152 SMs: 4 (3) CTAs are 2432 (1824) warps;
+# 768^2, 6 strips: items of 2 (3) rows, 2 (3) stages; 800^2, 7 strips: 3 (4) rows, 3 stages; 1024^2, 8 strips:
+# 4 (5) rows, 3 (4) stages; 1100^2, 9 strips: 5 (6) rows, 4 stages
+put("sms", 152)
+put("l2_kb", 129 << 10)
+fake.fake_device(2)
+for n, ctas_of in [(768, 6 * 384 / 4), (800, 7 * 200 / 4), (1024, 8 * 256 / 4), (1100, -(-9 * 184 // 4))]:
+    grid = solver("D2Q9", "LCDE", 2, [n, n], temporal_depth=1).step(1)[0][2]
+    assert grid == (ctas_of, 1, 1), (n, grid)
+put("sms", 4)
+put("l2_kb", 1024)
 put("ctas_per_sm", 2)                                  # a device with room for fewer (another one: kept per device)
 fake.fake_device(1)
 assert ctas("D2Q9", 2, [256, 800]) == 2
