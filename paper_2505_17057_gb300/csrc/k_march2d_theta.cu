@@ -2,15 +2,20 @@
 //
 // A step solves (I - (1 - theta) L) x = r, r = (I + theta L) phi^n, by Jacobi sweeps
 // x <- r / d + J x from x = phi^n (J: the sweep's stencil, no centre weight).  Two kernels:
-//   k_theta_first  one pass over phi^n writes r / d and the first sweep's result: that is
+//   k_theta_first  one pass over phi^n writes r and the first sweep's result: that is
 //                  r / d + J phi^n, one more linear stencil of phi^n.
 //   k_theta_sweeps TT further sweeps per launch, a wavefront of TT levels one row apart in registers as in
-//                  k_march2d_tb.  An output row's partial sum starts from its r / d, so the right-hand
-//                  side costs one load per row and launch and no addition.  The TT rows of it in use
-//                  sit in a register window indexed by the row modulo four (four rows per pass over
-//                  the loop, so no value moves), each fetched a row ahead of its use.
-// 4096^2 FP32, 17 sweeps, four per launch: 300 us a step; separate right-hand side pass, then sweeps adding the
-// right-hand side at the store, 369 us.  Bound by FP32 issue in the sweeps, by DRAM in the first pass.
+//                  k_march2d_tb.  The TT rows of r in use sit in a register window indexed by the row
+//                  modulo four (four rows per pass over the loop, so no value moves), each fetched a row
+//                  ahead of its use.  Two forms of a sweep:
+//     - an output row's partial sum starts from its r / d, rounded once: no addition in the sweep, but every
+//       term is then rounded at the full size of the sum;
+//     - the last sweeps of a step (the launches that hold one of its last four) sum J x first and add r (1 / d)
+//       at the end, as one fused operation: the rounding of the last sweeps is the step's error, that of
+//       earlier ones shrinks with every sweep after them.  With the first form throughout, a step's error
+//       against 64 bits was 1.1 to 2.2 times that of sweeps run one by one; with this rule the two agree.
+// 4096^2 FP32, 17 sweeps, four per launch: 296 us a step (317 with the second form throughout); separate
+// right-hand side pass, then sweeps adding the right-hand side at the store, 369 us.  Bound by FP32 issue in the sweeps, by DRAM in the first pass.
 // A row's sums of rows r (c) and r + 1 (n) are chains of fused multiply-adds on the sum of the row
 // before, with no accumulator copied from one role to the next.
 #include "k_march2d.cuh"
@@ -66,12 +71,12 @@ struct RowBox {
 };
 
 // FIRST: k_theta_first (TT = 1; rhs is written, A its stencil, and B gives the first sweep's result);
-// else the sweeps (rhs is read, B is J).
-template <int LAT, int ST, int TT, bool FIRST, int NW>
+// else the sweeps (rhs is read, B is J, jw is 1 / d; END: rhs is added at the end of a row's sum).
+template <int LAT, int ST, int TT, bool FIRST, bool END, int NW>
 __global__ void __launch_bounds__(NW * 32, ST == ST_F32 ? 4 : 1)
     k_theta(const __grid_constant__ TmapSet maps, Geom g, typename Storage<ST>::S* out,
             typename Storage<ST>::S* rhs, const __grid_constant__ Stencil<typename Storage<ST>::T> A,
-            const __grid_constant__ Stencil<typename Storage<ST>::T> B, int H, int nitems, int* err) {
+            const __grid_constant__ Stencil<typename Storage<ST>::T> B, typename Storage<ST>::T jw, int H, int nitems, int* err) {
     using S = typename Storage<ST>::S;
     using T = typename Storage<ST>::T;
     using X = RowBox<ST>;
@@ -172,14 +177,19 @@ __global__ void __launch_bounds__(NW * 32, ST == ST_F32 ? 4 : 1)
 #pragma unroll
             for (int k = 0; k < LN; ++k) ca[k] = na[k] = T(0);
         } else {
-            // the rows the first two input rows start (input row i starts row i + 1); earlier ones feed no output
+            // the first rows in use, by their place among the item's input rows: level 0 starts row i + 1 with
+            // input row i, and completes (END) row i - 1; earlier rows feed no output
 #pragma unroll
             for (int q = 0; q < 4; ++q)
 #pragma unroll
                 for (int k = 0; k < LN; ++k) win[q][k] = T(0);
-            ry = y0 - TT + 1;
+            ry = y0 - TT + (END ? 0 : 1);
             ry = ry < 0 ? ry + g.ny : ry % g.ny;
-            fetch(xb, win[1]);
+            if constexpr (!END) {
+                fetch(xb, win[1]);
+#pragma unroll
+                for (int k = 0; k < LN; ++k) win[1][k] = rmul(jw, win[1][k]);
+            }
             fetch(xb, next);
         }
         for (int i = 0; i < nrows && !failed; i += 4) {
@@ -218,8 +228,8 @@ __global__ void __launch_bounds__(NW * 32, ST == ST_F32 ? 4 : 1)
                     T o[LN];
                     const int yo = y0 - 2 * TT + i + J;
                     const bool stored = i + J >= 2 * TT && i + J < hrows + 2 * TT;   // warp-uniform
+                    const T zero[LN] = {T(-0.0), T(-0.0), T(-0.0), T(-0.0)};
                     if constexpr (FIRST) {
-                        const T zero[LN] = {T(-0.0), T(-0.0), T(-0.0), T(-0.0)};
                         T r[LN];
                         stencil_row<LAT, T>(A.W0, A.Wp, A.Wm, raw, zero, ca, na, r);
                         stencil_row<LAT, T>(B.W0, B.Wp, B.Wm, raw, zero, c[0], n[0], o);
@@ -236,14 +246,20 @@ __global__ void __launch_bounds__(NW * 32, ST == ST_F32 ? 4 : 1)
                                 raw[0] = __shfl_up_sync(0xffffffffu, raw[LN], 1);
                                 raw[LN + 1] = __shfl_down_sync(0xffffffffu, raw[1], 1);
                             }
-                            // level t takes row i + J - t and starts row i + J - t + 1
-                            stencil_row<LAT, T>(B.W0, B.Wp, B.Wm, raw, win[(J - t + 5) & 3], c[t], n[t], o);
+                            // level t takes row i + J - t, starts row i + J - t + 1 and completes row i + J - t - 1
+                            if constexpr (END) {
+                                stencil_row<LAT, T>(B.W0, B.Wp, B.Wm, raw, zero, c[t], n[t], o);
+#pragma unroll
+                                for (int k = 0; k < LN; ++k) o[k] = rfma(jw, win[(J - t + 7) & 3][k], o[k]);
+                            } else {
+                                stencil_row<LAT, T>(B.W0, B.Wp, B.Wm, raw, win[(J - t + 5) & 3], c[t], n[t], o);
+                            }
 #pragma unroll
                             for (int k = 0; k < LN; ++k) raw[1 + k] = o[k];
                         }
-                        // the row that input row i + J + 1 starts, and the fetch of the one after it
+                        // the row that input row i + J + 1 starts (END: completes), and the fetch of the one after it
 #pragma unroll
-                        for (int k = 0; k < LN; ++k) win[(J + 2) & 3][k] = next[k];
+                        for (int k = 0; k < LN; ++k) win[(END ? J : J + 2) & 3][k] = END ? next[k] : rmul(jw, next[k]);
                         fetch(xb, next);
                     }
                     if (stored) {
@@ -278,13 +294,13 @@ Stencil<T> stencil_of(const void* block) {
     return s;
 }
 
-template <int LAT, int ST, int TT, bool FIRST>
+template <int LAT, int ST, int TT, bool FIRST, bool END>
 cudaError_t launch(const LaunchArgs& a) {
     using T = typename Storage<ST>::T;
     using S = typename Storage<ST>::S;
     constexpr int NW = 4;
     constexpr size_t smem = RowBox<ST>::smem(NW);
-    auto kern = k_theta<LAT, ST, TT, FIRST, NW>;
+    auto kern = k_theta<LAT, ST, TT, FIRST, END, NW>;
     static std::atomic<unsigned long long> known[kMaxDevices];
     Fit fit;
     const cudaError_t e = fit_of(kern, NW * 32, smem, known, &fit);
@@ -297,35 +313,42 @@ cudaError_t launch(const LaunchArgs& a) {
     const int nitems = strips * ((a.g.ny + H - 1) / H);
     const int blocks = (nitems + NW - 1) / NW;
     Stencil<T> A{}, B;
+    T jw = T(0);
     if constexpr (FIRST) {
-        A = stencil_of<T, SrcCoef>(a.coef2);
+        A = stencil_of<T, Coef>(a.coef);
         B = stencil_of<T, SrcCoef>(a.src_coef);
     } else {
         B = stencil_of<T, Coef>(a.coef);
+        jw = static_cast<const SrcCoef<T>*>(a.src_coef)->W0[0];
     }
     return launch_chained(kern, blocks < resident ? blocks : resident, NW * 32, smem, a.stream, a.chained, *a.maps, a.g,
-                          static_cast<S*>(a.out), static_cast<S*>(const_cast<void*>(a.src[0])), A, B, H, nitems, a.err);
+                          static_cast<S*>(a.out), static_cast<S*>(const_cast<void*>(a.src[0])), A, B, jw, H, nitems, a.err);
 }
 
-template <int LAT>
+template <int LAT, bool END>
 LaunchFn pick(int st, int depth) {
-    if (depth == 0) return st == ST_F64 ? launch<LAT, ST_F64, 1, true> : launch<LAT, ST_F32, 1, true>;
-    if (st == ST_F64) return depth == 1 ? launch<LAT, ST_F64, 1, false> : depth == 2 ? launch<LAT, ST_F64, 2, false> : nullptr;
+    if (st == ST_F64)
+        return depth == 1 ? launch<LAT, ST_F64, 1, false, END> : depth == 2 ? launch<LAT, ST_F64, 2, false, END> : nullptr;
     switch (depth) {
-    case 1: return launch<LAT, ST_F32, 1, false>;
-    case 2: return launch<LAT, ST_F32, 2, false>;
-    case 3: return launch<LAT, ST_F32, 3, false>;
-    case 4: return launch<LAT, ST_F32, 4, false>;
+    case 1: return launch<LAT, ST_F32, 1, false, END>;
+    case 2: return launch<LAT, ST_F32, 2, false, END>;
+    case 3: return launch<LAT, ST_F32, 3, false, END>;
+    case 4: return launch<LAT, ST_F32, 4, false, END>;
     }
     return nullptr;
+}
+template <int LAT>
+LaunchFn pick_end(int st, int depth, bool end) {
+    if (depth == 0) return st == ST_F64 ? launch<LAT, ST_F64, 1, true, false> : launch<LAT, ST_F32, 1, true, false>;
+    return end ? pick<LAT, true>(st, depth) : pick<LAT, false>(st, depth);
 }
 
 }  // namespace
 
-LaunchFn find_march2d_theta(int lat, int st, int depth) {
+LaunchFn find_march2d_theta(int lat, int st, int depth, bool end) {
     if (st == ST_BF16) return nullptr;
-    if (lat == LAT_D2Q5) return pick<LAT_D2Q5>(st, depth);
-    if (lat == LAT_D2Q9) return pick<LAT_D2Q9>(st, depth);
+    if (lat == LAT_D2Q5) return pick_end<LAT_D2Q5>(st, depth, end);
+    if (lat == LAT_D2Q9) return pick_end<LAT_D2Q9>(st, depth, end);
     return nullptr;
 }
 

@@ -30,7 +30,6 @@ struct LaunchArgs {
     int* err;             // device error flag (bounded waits that ran out)
     const void* src[2];   // source levels t, t - dt (solvers with source terms; else null)
     const void* src_coef; // SrcCoef<double> or SrcCoef<float> matching the storage type
-    const void* coef2 = nullptr; // first pass of a theta-scheme step: stencil of rhs / d (see find_march2d_theta)
     const void* cls = nullptr; // NcdeClass<double> or NcdeClass<float> (the NCDE class kernels)
     bool chained = false; // a step of a chain on one stream: launched to overlap its predecessor's end (launch.cuh)
 };
@@ -80,10 +79,11 @@ LaunchFn find_march2d_nse(int st, int depth);
 LaunchFn find_march2d_tb_nse(int st, int depth);
 int march2d_tb_nse_max_depth();
 // The 2D theta-scheme kernels (FP32 / FP64 levels).  depth 0: the first pass of a step, from phi^n (in0)
-// to rhs / d (written to src[0], stencil coef2) and the first sweep's result (out, stencil src_coef),
-// both SrcCoef blocks; depth >= 1: that many further sweeps (stencil coef, a Coef block; src[0] = rhs / d),
-// up to march2d_tb_max_depth(st).
-LaunchFn find_march2d_theta(int lat, int st, int depth);
+// to rhs (written to src[0], stencil coef, a Coef block) and the first sweep's result (out, stencil
+// src_coef, a SrcCoef block); depth >= 1: that many further sweeps (stencil coef, a Coef block; src[0] =
+// rhs, its weight 1 / d in src_coef's W0[0]), up to march2d_tb_max_depth(st).  `end` picks the form with
+// the rounding of single sweeps, for the last ones of a step (k_march2d_theta.cu).
+LaunchFn find_march2d_theta(int lat, int st, int depth, bool end = false);
 // The same with source terms in the store epilogue (src as for find_direct_src; LCDE / NCDE).
 LaunchFn find_march3d_src(int lat, int pde, int levels, int st, int src);
 // The 2D (D2Q9) and 3D (D3Q19) NCDE marching kernels in class form (NcdeClass, FP32 / FP64 storage, two or

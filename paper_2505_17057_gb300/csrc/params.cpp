@@ -646,25 +646,19 @@ int resolve(const mmfd_desc& d_in, Resolved& r, std::string* msg) {
         }
         std::memset(&r.ths_d, 0, sizeof(r.ths_d));
         r.ths_d.W0[0] = 1.0 / dg;
-        std::memset(&r.thq_d, 0, sizeof(r.thq_d));
         std::memset(&r.th1_d, 0, sizeof(r.th1_d));
-        r.thq_d.W0[0] = R.W0[0] / dg;
-        r.th1_d.W0[0] = r.thq_d.W0[0] + J.W0[0];
+        r.th1_d.W0[0] = R.W0[0] / dg + J.W0[0];
         for (int p = 0; p < NP; ++p) {
-            r.thq_d.Wp[0][p] = R.Wp[0][p] / dg;
-            r.thq_d.Wm[0][p] = R.Wm[0][p] / dg;
-            r.th1_d.Wp[0][p] = r.thq_d.Wp[0][p] + J.Wp[0][p];
-            r.th1_d.Wm[0][p] = r.thq_d.Wm[0][p] + J.Wm[0][p];
+            r.th1_d.Wp[0][p] = R.Wp[0][p] / dg + J.Wp[0][p];
+            r.th1_d.Wm[0][p] = R.Wm[0][p] / dg + J.Wm[0][p];
         }
-        const double* srcs[5] = {reinterpret_cast<const double*>(&r.thr_d), reinterpret_cast<const double*>(&r.thj_d),
-                                 reinterpret_cast<const double*>(&r.ths_d), reinterpret_cast<const double*>(&r.thq_d),
-                                 reinterpret_cast<const double*>(&r.th1_d)};
-        float* dsts[5] = {reinterpret_cast<float*>(&r.thr_f), reinterpret_cast<float*>(&r.thj_f),
-                          reinterpret_cast<float*>(&r.ths_f), reinterpret_cast<float*>(&r.thq_f),
-                          reinterpret_cast<float*>(&r.th1_f)};
+        const double* srcs[4] = {reinterpret_cast<const double*>(&r.thr_d), reinterpret_cast<const double*>(&r.thj_d),
+                                 reinterpret_cast<const double*>(&r.ths_d), reinterpret_cast<const double*>(&r.th1_d)};
+        float* dsts[4] = {reinterpret_cast<float*>(&r.thr_f), reinterpret_cast<float*>(&r.thj_f),
+                          reinterpret_cast<float*>(&r.ths_f), reinterpret_cast<float*>(&r.th1_f)};
         const size_t nc = sizeof(Coef<double>) / sizeof(double), ns = sizeof(SrcCoef<double>) / sizeof(double);
-        const size_t counts[5] = {nc, nc, ns, ns, ns};
-        for (int b = 0; b < 5; ++b)
+        const size_t counts[4] = {nc, nc, ns, ns};
+        for (int b = 0; b < 4; ++b)
             for (size_t i = 0; i < counts[b]; ++i) dsts[b][i] = (float)srcs[b][i];
     }
 

@@ -42,10 +42,9 @@ struct Resolved {
     Coef<float> thr_f, thj_f;
     SrcCoef<double> ths_d;
     SrcCoef<float> ths_f;
-    // the same for the fused 2D kernels, level-t stencils: rhs / d (thq) and the first sweep's result
-    // rhs / d + thj phi^n (th1), both of phi^n
-    SrcCoef<double> thq_d, th1_d;
-    SrcCoef<float> thq_f, th1_f;
+    // and for the fused 2D kernels the first sweep's result rhs / d + thj phi^n as one stencil of phi^n
+    SrcCoef<double> th1_d;
+    SrcCoef<float> th1_f;
 };
 
 // Returns MMFD_OK or an error code; *msg gets a human-readable reason on error.

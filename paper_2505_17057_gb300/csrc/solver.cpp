@@ -270,10 +270,10 @@ int solver_step(Solver* s, long long nsteps) {
             LaunchArgs a;
             int left = s->r.sweeps;
             if (s->fn_block && s->depth > 1) {
-                // fused kernels: one pass for rhs / d and the first sweep, then `depth` sweeps per launch
+                // fused kernels: one pass for rhs and the first sweep, then `depth` sweeps per launch
                 // (fewer, with the launcher's own work-item height, for the remainder)
                 solver_launch_args(s, a);
-                a.coef2 = f64 ? static_cast<const void*>(&s->r.thq_d) : static_cast<const void*>(&s->r.thq_f);
+                a.coef = f64 ? static_cast<const void*>(&s->r.thr_d) : static_cast<const void*>(&s->r.thr_f);
                 a.src_coef = f64 ? static_cast<const void*>(&s->r.th1_d) : static_cast<const void*>(&s->r.th1_f);
                 a.H = 0;
                 cudaError_t e = s->fn_rhs(a);
@@ -282,7 +282,8 @@ int solver_step(Solver* s, long long nsteps) {
                 for (--left; left > 0;) {
                     solver_launch_args(s, a);
                     const int did = left < s->depth ? left : s->depth;
-                    const LaunchFn f = did == s->depth ? s->fn_block : find_march2d_theta(s->r.lat, s->r.st, did);
+                    const bool end = left - did < 4;   // (k_march2d_theta.cu)
+                    const LaunchFn f = did == s->depth && !end ? s->fn_block : find_march2d_theta(s->r.lat, s->r.st, did, end);
                     if (did != s->depth) a.H = 0;
                     e = f(a);
                     if (e != cudaSuccess) return cuda_fail(e, "theta-scheme sweep kernel");
