@@ -18,8 +18,8 @@
 //   current to the ghost depth.
 //
 // Bound by FP32 issue when blocked (46 instructions per node and step, the FMA pipe 64% busy), by DRAM with
-// one step per launch.  4096^2 FP32: three steps per launch 35.2 us per step (the pushed form 39.1), one
-// 75 us (77); FP64, bound by the FP64 rate, 1000 x 800 108 us (193).
+// one step per launch.  4096^2 FP32: three steps per launch 34.1 us per step (the pushed form 39.1), one
+// 75 us (77); FP64, bound by the FP64 rate, 1000 x 800 105 us (193).
 // FP32 and FP64 storage; BF16 levels keep the pushed form and its rounding (k_march2d_tb_nse,
 // k_march2d).
 #define MMFD_PAIRED 1
@@ -211,7 +211,7 @@ cudaError_t launch_nse(const LaunchArgs& a) {
     const int nitems = strips * ((a.g.ny + H - 1) / H);
     const int blocks_needed = (nitems + NW - 1) / NW;
     const int grid = blocks_needed < resident ? blocks_needed : resident;
-    return launch_chained(kern, grid, NW * 32, smem, a.stream, a.chained, *a.maps, a.g, a.out, class_coef<LAT_D2Q9, T>(*static_cast<const Coef<T>*>(a.coef), 0), H,
+    return launch_chained(kern, grid, NW * 32, smem, a.stream, a.chained, *a.maps, a.g, a.out, class_coef<LAT_D2Q9, T>(*static_cast<const Coef<T>*>(a.coef), a.umom, 0), H,
                           nitems, a.err);
 }
 

@@ -7,9 +7,9 @@
 // neighbouring lanes.  Lanes 0 and 31 evaluate the strip's halo columns, all lanes following.
 //
 // FP32 takes it for widths that are not a multiple of four and below 128 columns (find_march_lean): 250^3
-// 163 us a step (the pushed form 301), 510 x 512^2 1132 (2062), 96^3 16.5 (k_direct 28.4).  136
+// 161 us a step (the pushed form 301), 510 x 512^2 1110 (2062), 96^3 16.4 (k_direct 28.4).  136
 // instructions per node; at 512^3 4.5 TB/s, waits on the planes and FP32 issue in equal parts.  FP64
-// 144^3, bound by the FP64 rate, 1335 us (5300).
+// 144^3, bound by the FP64 rate, 1333 us (5300).
 #define MMFD_PAIRED 1
 #include "march3d_ring.cuh"
 #include "nse_class.cuh"
@@ -121,7 +121,7 @@ cudaError_t launch(const LaunchArgs& a) {
     int H = 0, nitems = 0, grid = 0;
     march3d_split(a.g, TY, a.H, resident, false, &H, &nitems, &grid);
     return launch_chained(kern, grid, THREADS, smem, a.stream, a.chained, *a.maps, a.g, a.out,
-                          class_norm<T>(*static_cast<const Coef<T>*>(a.coef), 0), H, nitems, a.err);
+                          class_norm<T>(*static_cast<const Coef<T>*>(a.coef), a.umom, 0), H, nitems, a.err);
 }
 
 template <int ST, int TY, size_t BUDGET>

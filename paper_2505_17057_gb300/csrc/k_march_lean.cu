@@ -51,7 +51,7 @@ LaunchFn find_march_lean(int lat, int levels, int st, int lean, int nx, int rows
         if (dim == 2) return find_march2d_nse(st, 1);
         // In 3D the FP32 pushed kernel, with its producer warp, is the faster one where its stores are whole
         // vectors; class form against pushed, us per step: 512^3 1009 / 974, 384^3 566 / 420, 256^3 154 / 139,
-        // 128^3 25 / 25, but 510 x 512^2 1132 / 2062, 250^3 163 / 301, 131 x 128^2 52 / 86.  Below 128 columns
+        // 128^3 25 / 25, but 510 x 512^2 1110 / 2062, 250^3 161 / 301, 131 x 128^2 52 / 86.  Below 128 columns
         // only the class form marches (kClassMinNx).
         if (st == ST_F64 || nx < 128 || nx % 4 != 0) return find_march3d_nse(st, rows);
     }

@@ -30,6 +30,7 @@ struct LaunchArgs {
     int* err;             // device error flag (bounded waits that ran out)
     const void* src[2];   // source levels t, t - dt (solvers with source terms; else null)
     const void* src_coef; // SrcCoef<double> or SrcCoef<float> matching the storage type
+    double umom = 1.0;     // the NSE class kernels: factor of a uniform velocity in one step (Resolved::umom)
     const void* cls = nullptr; // NcdeClass<double> or NcdeClass<float> (the NCDE class kernels)
     bool chained = false; // a step of a chain on one stream: launched to overlap its predecessor's end (launch.cuh)
 };

@@ -10,7 +10,7 @@
 //     are needed as their sum (rho and the other momenta) and difference (u_x);
 //   - along the marching axis, the whole group that an input row (plane) sends to the row behind
 //     (P), to its own (C) or to the one ahead (N) enters that axis's momentum with one sign.
-// Against pushing each v_j into every accumulator (lean_push_sv) that is 43 instead of 58
+// Against pushing each v_j into every accumulator (lean_push_sv) that is 42 instead of 58
 // floating-point operations per D2Q9 node and step, no node is evaluated twice (the x neighbours'
 // sums come from the neighbouring lanes), and, the main gain, every operation but the six x-shifted
 // sums acts on the lane's columns (0, 1) and (2, 3) alike: FP32 runs them as paired instructions
@@ -30,12 +30,20 @@ template <typename T>
 struct ClassCoef {
     Pk<T> nA[2], nU[2], nk[2], no[2], mo[2];   // k: 0 axis pairs, 1 diagonal pairs; mo = -no
     Pk<T> nc[2];                               // rest: a0 rho + a+ f_0^eq = nc[0] rho + nc[1] |u|^2
-    Pk<T> nsm;                                 // kappa c / rho0
-    Pk<T> abr;                                 // ab0 / nsm
+    Pk<T> nsm, msm;                            // kappa c / rho0, and minus that
+    Pk<T> ab0;
 };
 
+// ab0 as the class forms take it: a uniform velocity comes out of one step times ab0 + k, k the sum of the
+// rounded odd coefficients, which should be umom; in FP32 ab0 takes up what their rounding left (LBGK at
+// d_0 = 1/3 drifted by 2e-8 a step without).
+template <typename T>
+T class_ab0(T ab0, double k, double umom) {
+    return sizeof(T) == 8 ? ab0 : (T)(umom - k);
+}
+
 template <int LAT, typename T>
-ClassCoef<T> class_coef(const Coef<T>& cf, int l) {
+ClassCoef<T> class_coef(const Coef<T>& cf, double umom, int l) {
     constexpr int DG = lat_dim(LAT);   // first diagonal pair
     ClassCoef<T> c;
     for (int k = 0; k < 2; ++k) {
@@ -47,7 +55,8 @@ ClassCoef<T> class_coef(const Coef<T>& cf, int l) {
         c.nc[k] = Pk<T>::fill(cf.nc[l][k]);
     }
     c.nsm = Pk<T>::fill(cf.nsm[l][0]);
-    c.abr = Pk<T>::fill(cf.ab0[l] / cf.nsm[l][0]);
+    c.msm = Pk<T>::fill(-cf.nsm[l][0]);
+    c.ab0 = Pk<T>::fill(class_ab0(cf.ab0[l], (double)cf.nsm[l][0] * (2.0 * cf.no[l][0] + 4.0 * (DG - 1) * cf.no[l][DG]), umom));
     return c;
 }
 
@@ -58,12 +67,12 @@ template <typename T>
 struct ClassNorm {
     T dU, gk, be, lam;
     T cR, cU;      // rest: (a0 rho + a+ f_0^eq) / nA_0 = cR rho + cU |u|^2
-    T fR, fM;      // nA_0, nsm nA_0
-    T abr;         // ab0 / fM
+    T fR, fM, fD;  // nA_0, nsm nA_0, nsm nA_1
+    T ab0;
 };
 
 template <typename T>
-ClassNorm<T> class_norm(const Coef<T>& cf, int l) {
+ClassNorm<T> class_norm(const Coef<T>& cf, double umom, int l) {
     ClassNorm<T> c;
     const T n0 = cf.nA[l][0];
     c.dU = cf.nU[l][0] / n0;
@@ -74,7 +83,8 @@ ClassNorm<T> class_norm(const Coef<T>& cf, int l) {
     c.cU = cf.nc[l][1] / n0;
     c.fR = n0;
     c.fM = cf.nsm[l][0] * n0;
-    c.abr = cf.ab0[l] / c.fM;
+    c.fD = cf.nsm[l][0] * cf.nA[l][1];
+    c.ab0 = class_ab0(cf.ab0[l], (double)c.fM * c.be * (2.0 + 6.0 * c.lam) + 2.0 * c.fD * c.be, umom);
     return c;
 }
 
@@ -104,8 +114,7 @@ __device__ __forceinline__ void shift_lr(const Pk<T> (&L)[2], const Pk<T> (&R)[2
 // ------------------------------------------------------------------ D2Q9, rows marched in y
 
 // Sums of the output rows around the current input row r: row r (it has had row r-1's N group and
-// its own C group; row r+1's P group completes it) and row r+1 (row r's N group only).  Momentum
-// sums are in units of nsm.
+// its own C group; row r+1's P group completes it) and row r+1 (row r's N group only).
 template <typename T>
 struct Row2 {
     Pk<T> rho[2], mx[2], my[2];   // after the C group
@@ -152,15 +161,17 @@ __device__ __forceinline__ void class_row2d(const ClassCoef<T>& c, RowPk<T, 3>& 
     for (int h = 0; h < 2; ++h) {
         const P sum = padd(s[h], pE[h]);
         out[0][h] = padd(acc.rho[h], sum);
-        out[1][h] = pmul(c.nsm, padd(acc.mx[h], d[h]));
-        out[2][h] = pmul(c.nsm, padd(acc.my[h], sum));
+        out[1][h] = pfma(c.nsm, d[h], acc.mx[h]);
+        out[2][h] = pfma(c.nsm, sum, acc.my[h]);
     }
     shift_lr<T>(cL, cR, s, d);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         acc.rho[h] = padd(padd(ctr[h], acc.ns[h]), s[h]);
-        acc.mx[h] = pfma(c.abr, in.f[1][h], padd(acc.nd[h], d[h]));
-        acc.my[h] = psub(pmul(c.abr, in.f[2][h]), acc.ns[h]);
+        // (nsm and ab0 as they are: momentum sums kept in units of nsm take ab0 / nsm, whose rounding comes on
+        // top of nsm's, and with it a uniform flow drifted up to four times as fast)
+        acc.mx[h] = pfma(c.nsm, padd(acc.nd[h], d[h]), pmul(c.ab0, in.f[1][h]));
+        acc.my[h] = pfma(c.msm, acc.ns[h], pmul(c.ab0, in.f[2][h]));
     }
     shift_lr<T>(nL, nR, s, d);
 #pragma unroll
@@ -197,8 +208,8 @@ __device__ __forceinline__ void diff4(const T (&a)[4], const T (&b)[4], Pk<T> (&
 
 // Sums of one output row in the output planes around the current input plane z: plane z (it has
 // had plane z-1's N group and its own C group; plane z+1's P group completes it) and plane z+1
-// (plane z's N group only), in units of nA_0 (momentum: nsm nA_0).  nx, ny are the N group's x and
-// y momentum in units of lam; its z momentum is minus its sum.
+// (plane z's N group only): the momenta as they are, rho and the N group in units of nA_0.  nx, ny are the N
+// group's x and y momentum in units of nA_1; its z momentum is minus its sum.
 template <typename T>
 struct Row3 {
     Pk<T> rho[2], mx[2], my[2], mz[2];
@@ -278,7 +289,8 @@ template <typename T>
 __device__ __forceinline__ void class_row3d(const ClassNorm<T>& c, RowPk<T, 4>& in, const T (&e)[4], const Sides3<T>& sd,
                                             int lane, Row3<T>& acc) {
     using P = Pk<T>;
-    const P gk = P::fill(c.gk), o = P::fill(c.be), m = P::fill(-c.be), lam = P::fill(c.lam), abr = P::fill(c.abr);
+    const P gk = P::fill(c.gk), o = P::fill(c.be), m = P::fill(-c.be), lam = P::fill(c.lam), ab0 = P::fill(c.ab0);
+    const P fM = P::fill(c.fM), mM = P::fill(-c.fM), fD = P::fill(c.fD);
     P cL[2], cR[2], pL[2], pR[2], pE[2], nL[2], nR[2], nE[2], ctr[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -317,9 +329,9 @@ __device__ __forceinline__ void class_row3d(const ClassNorm<T>& c, RowPk<T, 4>& 
     for (int h = 0; h < 2; ++h) {
         const P sum = pfma(lam, padd(s[h], sd.sP[h]), pE[h]);
         out[0][h] = pmul(P::fill(c.fR), padd(acc.rho[h], sum));
-        out[1][h] = pmul(P::fill(c.fM), pfma(lam, d[h], acc.mx[h]));
-        out[2][h] = pmul(P::fill(c.fM), pfma(lam, sd.dP[h], acc.my[h]));
-        out[3][h] = pmul(P::fill(c.fM), padd(acc.mz[h], sum));
+        out[1][h] = pfma(fD, d[h], acc.mx[h]);
+        out[2][h] = pfma(fD, sd.dP[h], acc.my[h]);
+        out[3][h] = pfma(fM, sum, acc.mz[h]);
     }
     shift_lr_edge<T>(sd.dL, sd.dR, sd.hd, lane, a, b);
     sum4<T>(a, b, y);
@@ -335,9 +347,9 @@ __device__ __forceinline__ void class_row3d(const ClassNorm<T>& c, RowPk<T, 4>& 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         acc.rho[h] = padd(padd(ctr[h], acc.ns[h]), padd(s[h], sd.sE[h]));
-        acc.mx[h] = pfma(abr, in.f[1][h], pfma(lam, acc.nx[h], d[h]));
-        acc.my[h] = pfma(abr, in.f[2][h], pfma(lam, padd(acc.ny[h], y[h]), sd.dE[h]));
-        acc.mz[h] = psub(pmul(abr, in.f[3][h]), acc.ns[h]);
+        acc.mx[h] = pfma(fM, pfma(lam, acc.nx[h], d[h]), pmul(ab0, in.f[1][h]));
+        acc.my[h] = pfma(fM, pfma(lam, padd(acc.ny[h], y[h]), sd.dE[h]), pmul(ab0, in.f[2][h]));
+        acc.mz[h] = pfma(mM, acc.ns[h], pmul(ab0, in.f[3][h]));
     }
     shift_lr_edge<T>(nL, nR, hN, lane, a, b);
     sum4<T>(a, b, s);

@@ -524,6 +524,8 @@ int resolve(const mmfd_desc& d_in, Resolved& r, std::string* msg) {
     }
     for (int f = 0; f < 4; ++f) c.ref[f] = r.ref[f];
     r.lean = (d.pde == PDE_NSE && !axis) ? nse_lean(c, d.lattice, dim, d.levels) : LEAN_NONE;
+    // (pairs that span an axis: the axis pair, and 2 (dim - 1) diagonal ones)
+    r.umom = r.lean == LEAN_STREAM ? c.ab0[0] + c.nsm[0][0] * (2.0 * c.no[0][0] + 4.0 * (dim - 1) * c.no[0][dim]) : 1.0;
 
     r.ncls = NCLS_NONE;
     std::memset(&r.ncd, 0, sizeof(r.ncd));

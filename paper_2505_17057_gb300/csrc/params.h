@@ -26,6 +26,7 @@ struct Resolved {
     NcdeClass<double> ncd;
     NcdeClass<float> ncf;
     int lean;           // LEAN_*: lean He-Luo form available to the marching kernels
+    double umom;        // LEAN_STREAM, two levels: factor of a uniform velocity in one step (1 for a scheme that keeps it)
     int src;            // MMFD_SRC_* (0: none)
     int nsrc;           // source fields per level (S, then M_1F components)
     double b[3], bhat[3];

@@ -358,6 +358,7 @@ int launch_tick(Server* s) {
         a.in1 = nl == 3 ? q->lev[prev] : nullptr;
         a.out = q->lev[next];
         a.coef = q->r->st == ST_F64 ? static_cast<const void*>(&q->r->cd) : static_cast<const void*>(&q->r->cf);
+        a.umom = q->r->umom;
         a.ex.seed = q->desc.seed;
         a.ex.step = step0 + steps;
         a.ex.sr = (q->r->st == ST_BF16 && (q->desc.flags & MMFD_FLAG_STOCHASTIC_ROUND)) ? 1 : 0;

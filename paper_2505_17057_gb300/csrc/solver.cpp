@@ -211,6 +211,7 @@ void solver_launch_args(Solver* s, LaunchArgs& a) {
     a.in1 = s->nlev == 3 ? s->lev[s->prev()] : nullptr;
     a.out = s->lev[s->next()];
     a.coef = s->coef();
+    a.umom = s->r.umom;
     a.ex.seed = s->desc.seed;
     a.ex.step = s->steps_done + 1;
     a.ex.sr = (s->r.st == ST_BF16 && (s->desc.flags & MMFD_FLAG_STOCHASTIC_ROUND)) ? 1 : 0;
