@@ -535,6 +535,20 @@ int resolve(const mmfd_desc& d_in, Resolved& r, std::string* msg) {
         float* dst = reinterpret_cast<float*>(&r.ncf);
         static_assert(sizeof(NcdeClass<double>) == 2 * sizeof(NcdeClass<float>), "NcdeClass layout");
         for (size_t i = 0; i < sizeof(NcdeClass<double>) / sizeof(double); ++i) dst[i] = (float)src[i];
+        // A uniform phi gets the sum of a level's coefficients, whose roundings would make it drift by 1e-8 a step
+        // and more: the diagonal pairs' take up what the others' rounding left, and the axis pairs' (finer
+        // where they vanish, as M2's do on D3Q19 with d_0 = 1/3) what is left then.  (2 dim axis directions,
+        // 2 dim (dim - 1) diagonal ones.)
+        const double na = 2.0 * dim, nd = 2.0 * dim * (dim - 1);
+        auto keep_sum = [&](double rest, const double* e, float restf, float* ef) {
+            const double sum = rest + na * e[0] + nd * e[1];
+            ef[1] = (float)((sum - restf - na * ef[0]) / nd);
+            ef[0] = (float)((sum - restf - nd * ef[1]) / na);
+        };
+        for (int l = 0; l < d.levels - 1 && r.ncls != NCLS_NONE; ++l) {
+            keep_sum(r.ncd.cP[l], r.ncd.eP[l], r.ncf.cP[l], r.ncf.eP[l]);
+            keep_sum(r.ncd.cM[l], r.ncd.eM[l], r.ncf.cM[l], r.ncf.eM[l]);
+        }
     }
 
     // float copy

@@ -63,3 +63,18 @@ def test_nse(mm, monkeypatch, lat, n, d0, steps, a0):
     cls, gen = errors(mm, monkeypatch, kw, steps,
                       lambda rng, sh: [1.0 + modes(rng, sh, 0.01)] + [modes(rng, sh, 0.05) for _ in range(dim)])
     assert np.all(cls <= 1.1 * gen), (cls, gen)
+
+
+@pytest.mark.parametrize("a", [(0.95, 0.1, -0.05), (0.8, 0.4, -0.2), None])
+@pytest.mark.parametrize("lat,n", [("D2Q9", [200, 160]), ("D3Q19", [130, 40, 36])])
+@pytest.mark.parametrize("shared", [True, False])
+def test_ncde(mm, monkeypatch, lat, n, a, shared):
+    dim = len(n)
+    kw = dict(pde="NCDE", lattice=lat, n=n, dt=0.8, dx=[1.0] * dim, diff=[0.15, 0, 0.05, 0],
+              flux=([[0, 0.05, 0.1, 0]] * 3 if shared else [[0, 0.05, 0.1, 0], [0, -0.03, 0.1, 0], [0, 0, 0.06, 0.02]])[:dim])
+    if a:
+        kw.update(levels=2, a=a)
+    else:
+        kw.update(levels=3, a=(7 / 8, 0.0, 1 / 8), ahat=(1 / 8, 0.0, -1 / 8))
+    cls, gen = errors(mm, monkeypatch, kw, 40, lambda rng, sh: [0.5 + modes(rng, sh, 0.2)])
+    assert np.all(cls <= 1.1 * gen), (cls, gen)
