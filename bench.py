@@ -15,6 +15,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -68,38 +69,51 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-# Sources that determine each step kernel's code and launch shape -- the kernel, its launcher,
-# the autotuner that picks the work-item height and the tensor-map boxes (the traffic figure of
-# a committed profile is used only while these files are unchanged).
+# The sources that determine the step kernels a solver may run under each kernel name it reports (the
+# family's name: FP32 levels of the NSE families, FP64 levels and NCDE solves run kernels of their own in
+# class form), and their launches.  The traffic figure of a committed profile is used only while
+# these files and everything they include are unchanged.
+COMMON_SOURCES = ["tune.cpp", "tma_host.cpp", "params.cpp"]   # work-item heights, tensor-map boxes, which form applies
 KERNEL_SOURCES = {
-    "k_march2d": ["k_march2d.cuh", "k_march2d.cu", "stencil.cuh", "tma.cuh", "mmfd_internal.h", "kernels.h",
-                  "k_direct.cuh", "tune.cpp", "tma_host.cpp"],
-    "k_march2d_tb": ["k_march2d_tb.cu", "k_march2d.cuh", "stencil.cuh", "tma.cuh", "mmfd_internal.h", "kernels.h",
-                     "k_direct.cuh", "tune.cpp", "tma_host.cpp"],
-    "k_march3d": ["k_march3d.cuh", "k_march3d.cu", "k_march2d.cuh", "stencil.cuh", "tma.cuh", "mmfd_internal.h",
-                  "kernels.h", "k_direct.cuh", "tune.cpp", "tma_host.cpp"],
-    # the lean He-Luo NSE variants (streaming / general momentum) of the marching kernels
-    "k_march2d_nse_s": ["k_march_lean.cu", "k_march2d.cuh", "stencil.cuh", "tma.cuh", "mmfd_internal.h", "kernels.h",
-                        "k_direct.cuh", "tune.cpp", "tma_host.cpp", "params.cpp"],
-    "k_march3d_nse_s": ["k_march_lean.cu", "k_march3d.cuh", "k_march2d.cuh", "stencil.cuh", "tma.cuh",
-                        "mmfd_internal.h", "kernels.h", "k_direct.cuh", "tune.cpp", "tma_host.cpp", "params.cpp"],
-    "k_march2d_tb_nse": ["k_march2d_tb_nse.cu", "k_march2d.cuh", "stencil.cuh", "tma.cuh", "mmfd_internal.h",
-                         "kernels.h", "k_direct.cuh", "tune.cpp", "tma_host.cpp", "params.cpp"],
-    "k_march2d_src": ["k_march2d_src.cu", "k_march2d.cuh", "stencil.cuh", "tma.cuh", "mmfd_internal.h", "kernels.h",
-                      "k_direct.cuh", "tune.cpp", "tma_host.cpp"],
-    # one theta-scheme step: the right-hand side (k_march2d) and the Jacobi sweeps (k_march2d_tb
-    # fusing several per launch, k_march2d_src for single ones), issued by solver.cpp; the traffic
-    # entry also records the sweep count it was taken at
-    "k_march2d_theta": ["k_march2d_src.cu", "k_march2d.cu", "k_march2d_tb.cu", "k_march2d.cuh", "stencil.cuh", "tma.cuh",
-                        "mmfd_internal.h", "kernels.h", "k_direct.cuh", "tune.cpp", "tma_host.cpp", "solver.cpp"],
+    "k_march2d": ["k_march2d.cu", "k_march2d_nse.cu", "k_march_ncde.cu"],
+    "k_march2d_tb": ["k_march2d_tb.cu"],
+    "k_march2d_nse_s": ["k_march_lean.cu", "k_march2d_nse.cu"],
+    "k_march2d_nse_g": ["k_march_lean.cu"],
+    "k_march2d_tb_nse": ["k_march2d_tb_nse.cu", "k_march2d_nse.cu"],
+    "k_march2d_src": ["k_march2d_src.cu"],
+    "k_march3d": ["k_march3d.cu", "k_march3d_nse.cu", "k_march_ncde.cu"],
+    "k_march3d_nse_s": ["k_march_lean.cu", "k_march3d_nse.cu"],
+    "k_march3d_nse_g": ["k_march_lean.cu"],
+    "k_march3d_src": ["k_march3d_src.cu"],
+    "k_direct": ["k_direct.cu", "k_cluster.cu"],
+    "k_direct_src": ["k_direct_src.cu"],
+    # one theta-scheme step: the first pass and the fused sweeps, or the right-hand side and single sweeps,
+    # issued by solver.cpp; the traffic entry also records the sweep count it was taken at
+    "k_march2d_theta": ["k_march2d_theta.cu", "k_march2d_src.cu", "k_march2d.cu", "solver.cpp"],
 }
+CSRC = os.path.join(ROOT, "paper_2505_17057_gb300", "csrc")
+
+
+def kernel_sources(kernel: str):
+    """The source files of a kernel name, with everything they include (sorted; all files for an unknown name)."""
+    todo = list(COMMON_SOURCES) + KERNEL_SOURCES.get(kernel, [f for f in os.listdir(CSRC)])
+    seen = set()
+    while todo:
+        f = todo.pop()
+        if f in seen:
+            continue
+        seen.add(f)
+        with open(os.path.join(CSRC, f)) as fh:
+            for inc in re.findall(r'^\s*#\s*include\s+"([^"]+)"', fh.read(), flags=re.M):
+                if os.path.exists(os.path.join(CSRC, inc)):
+                    todo.append(inc)
+    return sorted(seen)
 
 
 def kernel_source_sha(kernel: str) -> str:
     h = hashlib.sha256()
-    csrc = os.path.join(ROOT, "paper_2505_17057_gb300", "csrc")
-    for f in sorted(KERNEL_SOURCES.get(kernel, os.listdir(csrc))):
-        with open(os.path.join(csrc, f), "rb") as fh:
+    for f in kernel_sources(kernel):
+        with open(os.path.join(CSRC, f), "rb") as fh:
             h.update(f.encode() + fh.read())
     return h.hexdigest()[:16]
 
