@@ -59,11 +59,13 @@ def test_sources_are_closed_under_includes(name):
 
 def test_a_header_changes_the_hash(monkeypatch, tmp_path):
     import shutil
-    shutil.copytree(CSRC, tmp_path / "csrc")
+    base = tmp_path / "pkg"                       # the headers beside the package are included by relative path
+    shutil.copytree(CSRC, base / "csrc")
+    shutil.copytree(os.path.join(ROOT, "include"), tmp_path / "include")
     before = {k: bench.kernel_source_sha(k) for k in RUNS}
-    monkeypatch.setattr(bench, "CSRC", str(tmp_path / "csrc"))
+    monkeypatch.setattr(bench, "CSRC", str(base / "csrc"))
     assert {k: bench.kernel_source_sha(k) for k in RUNS} == before
-    with open(tmp_path / "csrc" / "nse_class.cuh", "a") as fh:
+    with open(base / "csrc" / "nse_class.cuh", "a") as fh:
         fh.write("\n")
     after = {k: bench.kernel_source_sha(k) for k in RUNS}
     assert {k for k in RUNS if after[k] != before[k]} == {"k_march2d", "k_march2d_nse_s", "k_march2d_tb_nse", "k_march3d",
