@@ -207,7 +207,10 @@ typedef struct {
     long long device_bytes;      /* device memory held by the level buffers */
     int temporal_depth;          /* depth in use */
     long long steps_done;        /* time levels advanced so far */
-    char kernel[32];             /* name of the step kernel family in use */
+    char kernel[32];             /* name of the step kernel family in use, whatever form its kernels take: the
+                                    class forms of the NSE and NCDE steps go by the names of the kernels
+                                    they stand in for (k_march2d_nse_s, k_march2d_tb_nse, k_march2d, ...), the
+                                    fused theta-scheme sweeps by k_march2d_tb, the cluster kernel by k_direct */
     int sweeps;                  /* theta-scheme: Jacobi sweeps per step (0: explicit scheme) */
     int tile_rows;               /* 3D marching kernels: rows of the x-y tile a CTA stages per plane
                                     (16 for the lean NSE kernels on large grids, else 4 or 8); 0 for

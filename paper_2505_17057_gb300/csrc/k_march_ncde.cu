@@ -7,7 +7,7 @@
 // 3D: the tiles, ring and refill of k_march3d_nse; a warp owns R output rows and evaluates each of
 // its R + 2 input rows once per plane, lanes 0 and 31 also the strip's halo columns.
 //
-// Bound by FP32 (FP64) issue.  Shared flux, two levels: 2D 4096^2 FP32 42.5 us a step (the pushed form 74.6),
+// Bound by FP32 (FP64) issue.  Shared flux, three levels: 2D 4096^2 FP32 42.5 us a step (the pushed form 74.6),
 // 1024^2 5.8 us (10.6), FP64 151 us (389); 3D 96^3 FP32 13.4 us (22.9), 256^3 118 us (227), FP64 96^3 409 us
 // (979).
 #define MMFD_PAIRED 1

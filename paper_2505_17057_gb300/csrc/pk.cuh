@@ -1,5 +1,7 @@
-// pk.cuh -- arithmetic on two neighbouring nodes at once, every operation rounded as written (one
-// rounding per multiply, add or fused multiply-add).
+// pk.cuh -- arithmetic on one node, or on two neighbouring nodes at once, every operation rounded as written:
+// one rounding per multiply, add or fused multiply-add, none left to the compiler's choice of
+// contraction.  Kernels that evaluate the same node's contributions in different contexts (a value with one
+// use in one kernel, two in another) then round alike.
 //
 // MMFD_PAIRED, set by a source file before its includes, picks the FP32 form.  1: paired instructions
 // (fma.f32x2 and the like), one issue slot for both nodes, at the price of register pairs for the

@@ -199,10 +199,6 @@ __device__ __forceinline__ T edot(T ux, T uy, T uz) {
 // General: sE = a+ E and mO = abar+ O (formed once per pair and node), the scalar contribution
 // a- O +- ... and the momentum abar- E +- ... of Eq. (2-4-1) as in the general pair form.
 // acc points at the output node's NF accumulators.
-// Arithmetic with its rounding fixed by the source: one rounding per multiply, add or fused
-// multiply-add, none left to the compiler's choice of contraction.  Kernels that evaluate the same
-// node's contributions in different contexts (a value with one use in one kernel, two in another)
-// then round alike.
 
 // Streaming momentum: a contribution sv of pair P in direction SIGN into one output node's
 // accumulators (scalar sv, momentum +-kappa c_a / rho0 times sv).
